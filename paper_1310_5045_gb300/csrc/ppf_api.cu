@@ -60,7 +60,7 @@ void free_all(ppf_ctx *c)
 {
     void *ptrs[] = {c->tang[0], c->tang[1], c->gpart,
                     c->state[0], c->state[1], c->anc, c->anc_sys, c->lwp, c->goff, c->goff_new, c->ring, c->succ, c->Zp,
-                    c->frame_buf[0], c->frame_buf[1], c->lmap, c->part, c->sum, c->est_dev, c->sc.Qt, c->sc.Ct, c->sc.Tt, c->sc.item_off, c->sc.extra, c->sc.Cbl,
+                    c->frame_buf[0], c->frame_buf[1], c->lmap, c->part, c->sum, c->est_dev, c->sc.Qt, c->sc.St, c->sc.Ct, c->sc.Tt, c->sc.To, c->sc.extra, c->sc.Cbl,
                     c->sc.Tg, c->sc.tile_g, c->sc.ggrid, c->sc.split, c->sc.skey, c->sc.sval, c->sc.seg_tick, c->sc.seg_dst, c->sc.seg_len,
                     c->sc.seg_chunk, c->bin_key, c->bin_l, c->bin_tot, c->bin_item, c->bin_rec};
     for (void *p : ptrs)
@@ -226,9 +226,10 @@ ppf_status ppf_create(const ppf_model *m, int64_t n, int32_t group_size, void *s
         chk(dalloc(&c->sum, 1), "summary");
         chk(dalloc(&c->est_dev, 1), "estimate staging");
         chk(dalloc(&c->sc.Qt, T), "Qt");
+        chk(dalloc(&c->sc.St, 8 * T), "St");
         chk(dalloc(&c->sc.Ct, T + 1), "Ct");
         chk(dalloc(&c->sc.Tt, T + 1), "Tt");
-        chk(dalloc(&c->sc.item_off, T + 1), "item_off");
+        chk(dalloc(&c->sc.To, T), "To");
         chk(dalloc(&c->sc.extra, 2 * (N / ppf::ITEM_TICKETS + 1)), "further runs");
         chk(dalloc(&c->sc.Cbl, G + 1), "Cbl");
         chk(dalloc(&c->sc.Tg, G + 1), "Tg");
@@ -387,6 +388,9 @@ ppf_status ppf_resample_if(ppf_ctx *c, ppf_scheme scheme, float alpha, double es
     } else {
         CK(ppf::launch_resample_global(c, (int)scheme, ess_threshold));
         if (scheme != PPF_SYSTEMATIC) {
+            // GS and SGS leave the balanced layout (unless the N_eff test or
+            // degenerate weights keep the groups as they are)
+            c->uneven = c->uneven || scheme == PPF_RPA_LGS || scheme == PPF_RPA2_LGS;
             int64_t *t = c->goff;
             c->goff = c->goff_new;
             c->goff_new = t;
@@ -544,6 +548,7 @@ ppf_status ppf_set_groups(ppf_ctx *c, const int64_t *offsets_host)
     CK(cudaStreamSynchronize(c->stream));  // offsets_host may be released on return
     CK(store_group_extents(c, offsets_host));
     CK(identity_ring(c));
+    c->uneven = true;
     return PPF_OK;
 }
 

@@ -93,8 +93,11 @@ struct ppf_batch {
     int32_t *tile_n;
     int32_t *ft_off;                   // device [F + 1]: tiles of filter f
     uint64_t *tQ;                      // device [T] tile totals
+    uint64_t *tS;                      // device [8T]: the weight below each strip of the tile
     uint64_t *tC;                      // device [T] exclusive prefix within the filter
     int64_t *tT;                       // device [T + 1]: first ticket of the tile (filter-local)
+    int32_t *tO;                       // device [T]: run_offset of the tile's tickets
+    int4 *fsc;                         // device [F]: the ticket counts' scale (TicketScale)
     uint64_t *fQu;                     // device [4F]: per filter Q_f, u_f, Q_f / n_f, Q_f mod n_f
     ppf::Partial *upart;               // device [U]
     ppf::FilterSummary *fsum;          // device [F]
@@ -367,9 +370,10 @@ __global__ void __launch_bounds__(TILE_THREADS) batch_tile_totals(const float *s
                                                                   const int32_t *__restrict__ tile_f,
                                                                   const int64_t *__restrict__ tile_lo,
                                                                   const int32_t *__restrict__ tile_n,
-                                                                  uint64_t *__restrict__ tQ)
+                                                                  uint64_t *__restrict__ tQ,
+                                                                  uint64_t *__restrict__ tS)
 {
-    __shared__ uint64_t red[33];
+    __shared__ uint64_t red[STRIPS];
     const float *__restrict__ lw = (cur->cur ? st0 : st1) + 5 * Ntot;
     const int32_t t = blockIdx.x, f = tile_f[t];
     if (fs[f].ess >= fp[f].ess_thr)
@@ -379,29 +383,30 @@ __global__ void __launch_bounds__(TILE_THREADS) batch_tile_totals(const float *s
     const int n = tile_n[t];
     const float *__restrict__ w = lw + tile_lo[t];
     // all loads first (independent, in flight together), then the quantiser
-    float v[TILE_ITEMS];
-#pragma unroll
-    for (int k = 0; k < TILE_ITEMS; ++k) {
-        const int i = threadIdx.x + k * TILE_THREADS;
-        v[k] = (i < n) ? __ldg(w + i) : -INFINITY;
-    }
     uint64_t acc = 0;
+    if ((int)(threadIdx.x >> 5) * (TILE / STRIPS) < n) {  // not a strip beyond the tile's end
+        float v[TILE_ITEMS];
+        strip_load(w, n, v);
 #pragma unroll
-    for (int k = 0; k < TILE_ITEMS; k += 2) {
-        uint64_t a, b;
-        quantise2(v[k], v[k + 1], Mf, s, a, b);
-        acc += a + b;
+        for (int k = 0; k < TILE_ITEMS; k += 2) {
+            uint64_t a, b;
+            quantise2(v[k], v[k + 1], Mf, s, a, b);
+            acc += a + b;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            acc += __shfl_xor_sync(0xffffffffu, acc, o);
     }
-    uint64_t total;
-    block_excl_scan_u64(acc, red, &total);
-    if (threadIdx.x == 0)
-        tQ[t] = total;
+    if ((threadIdx.x & 31) == 0)
+        red[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    store_strips(red, tS + (int64_t)t * STRIPS, tQ + t);
 }
 
 __global__ void batch_tile_scan(const FilterParams *__restrict__ fp, const FilterSummary *__restrict__ fs,
                                 const BatchCursor *__restrict__ cur, const int32_t *__restrict__ ft_off, int32_t F,
                                 const uint64_t *__restrict__ tQ, uint64_t *__restrict__ tC, int64_t *__restrict__ tT,
-                                uint64_t *__restrict__ fQu, int32_t *__restrict__ fkeep, int32_t *__restrict__ flags)
+                                int32_t *__restrict__ tO, int4 *__restrict__ fsc, uint64_t *__restrict__ fQu, int32_t *__restrict__ fkeep, int32_t *__restrict__ flags)
 {
     const int32_t f = (int32_t)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
@@ -432,6 +437,10 @@ __global__ void batch_tile_scan(const FilterParams *__restrict__ fp, const Filte
         fQu[4 * f + 1] = u;
         fQu[4 * f + 2] = Q / (uint64_t)P.n;
         fQu[4 * f + 3] = Q % (uint64_t)P.n;
+        if (Q != 0ull) {  // and the ticket counts' scale
+            const TicketScale sc = ticket_scale(Q, (uint32_t)P.n);
+            fsc[f] = make_int4((int32_t)sc.v, sc.sr, sc.sl, 0);
+        }
         fkeep[f] = (Q == 0ull) ? 1 : 0;  // no usable weight: kept as well
         if (Q == 0ull)
             atomicOr(flags, FLAG_DEGENERATE);
@@ -442,11 +451,16 @@ __global__ void batch_tile_scan(const FilterParams *__restrict__ fp, const Filte
         return;
     }
     const TicketGrid tg = ticket_grid(Q, u, Q / (uint64_t)P.n, (uint32_t)(Q % (uint64_t)P.n), P.ndiv);
-    for (int32_t t = t0 + lane; t < t1; t += 32)
-        tT[t] = tickets_below_grid(tC[t], tg);
+    const TicketScale sc = ticket_scale(Q, (uint32_t)P.n);
+    for (int32_t t = t0 + lane; t < t1; t += 32) {
+        const uint64_t c = tC[t];
+        const int64_t j = tickets_below_grid(c, tg);
+        tT[t] = j;
+        tO[t] = run_offset(c, tg, sc, j, true);
+    }
 }
 
-__global__ void __launch_bounds__(TILE_THREADS) batch_fill(const float *st0, const float *st1, int64_t Ntot,
+__global__ void __launch_bounds__(TILE_THREADS, 4) batch_fill(const float *st0, const float *st1, int64_t Ntot,
                                                            const FilterParams *__restrict__ fp,
                                                            const FilterSummary *__restrict__ fs,
                                                            const BatchCursor *__restrict__ cur,
@@ -456,13 +470,13 @@ __global__ void __launch_bounds__(TILE_THREADS) batch_fill(const float *st0, con
                                                            const int32_t *__restrict__ ft_off,
                                                            const uint64_t *__restrict__ tC,
                                                            const int64_t *__restrict__ tT,
+                                                           const int32_t *__restrict__ tO,
+                                                           const uint64_t *__restrict__ tS,
+                                                           const int4 *__restrict__ fsc,
                                                            const uint64_t *__restrict__ fQu, int32_t *__restrict__ anc,
                                                            int32_t *flags)
 {
-    extern __shared__ uint64_t fill_smem[];  // FILL_SMEM_BYTES
-    uint64_t *C = fill_smem;
-    uint16_t *stage = reinterpret_cast<uint16_t *>(fill_smem + TILE_SMEM_U64);
-    __shared__ uint64_t red[33];
+    __shared__ ParentSmem sm;
     const float *__restrict__ lw = (cur->cur ? st0 : st1) + 5 * Ntot;
     const int32_t t = blockIdx.x, f = tile_f[t];
     const FilterParams P = fp[f];
@@ -477,12 +491,23 @@ __global__ void __launch_bounds__(TILE_THREADS) batch_fill(const float *st0, con
     const int32_t tl = ft_off[f + 1] - 1;
     const int64_t j_lo = tT[t];
     const int64_t j_hi = (t < tl) ? tT[t + 1] : P.n;
-    uint64_t q[TILE_ITEMS];
-    tile_weights(lw, lo, n, fs[f].M, scale_bits(P.n), C, q);
-    tile_scan(q, C, red);
+    const int64_t j_max = (P.n < Ntot - P.off) ? P.n : Ntot - P.off;
     const TicketGrid tg = ticket_grid(Q, u, fQu[4 * f + 2], (uint32_t)fQu[4 * f + 3], P.ndiv);
-    ticket_parents_contig(C, n, tC[t], tg, j_lo, j_hi, stage, anc + P.off, (int32_t)lo,
-                          (P.n < Ntot - P.off) ? P.n : Ntot - P.off, flags);
+    const int4 q4 = fsc[f];
+    const TicketScale sc{(uint32_t)q4.x, q4.y, q4.z};
+    const float M = fs[f].M;
+    const int s = scale_bits(P.n);
+    const uint64_t below = tS[(int64_t)t * STRIPS + (threadIdx.x >> 5)];
+    auto sums = [&](TileSums &t1) {
+        float v[TILE_ITEMS];
+        tile_load16(lw, Ntot, lo, n, v);
+        tile_quantise(v, M, s, t1);
+        strip_scan(t1, below);
+    };
+    TileSums ts;
+    sums(ts);
+    draw_parents(ts, tC[t], tg, sc, j_lo, j_hi, true, tO[t], sm, EmitContig{anc + P.off, (int32_t)lo, n, j_max, flags},
+                 sums);
 }
 
 // ------------------------------------------------------------------ host side
@@ -549,6 +574,9 @@ cudaError_t build_tiles(ppf_batch *b)
     if ((e = dmalloc(&b->tQ, b->T)) != cudaSuccess) return e;
     if ((e = dmalloc(&b->tC, b->T)) != cudaSuccess) return e;
     if ((e = dmalloc(&b->tT, b->T + 1)) != cudaSuccess) return e;
+    if ((e = dmalloc(&b->tS, STRIPS * (size_t)b->T)) != cudaSuccess) return e;
+    if ((e = dmalloc(&b->fsc, b->F)) != cudaSuccess) return e;
+    if ((e = dmalloc(&b->tO, b->T)) != cudaSuccess) return e;
     if ((e = dmalloc(&b->fQu, 4 * (size_t)b->F)) != cudaSuccess) return e;
     if ((e = cudaMemcpy(b->tile_f, tf.data(), sizeof(int32_t) * b->T, cudaMemcpyHostToDevice)) != cudaSuccess) return e;
     if ((e = cudaMemcpy(b->tile_lo, tl.data(), sizeof(int64_t) * b->T, cudaMemcpyHostToDevice)) != cudaSuccess) return e;
@@ -639,12 +667,12 @@ cudaError_t set_cursor(ppf_batch *b, const void *frames, FilterSummary *est, int
 cudaError_t launch_batch_resample(ppf_batch *b)
 {
     batch_tile_totals<<<b->T, TILE_THREADS, 0, b->stream>>>(b->state[0], b->state[1], b->Ntot, b->fp, b->fsum,
-                                                            b->cursor, b->tile_f, b->tile_lo, b->tile_n, b->tQ);
+                                                            b->cursor, b->tile_f, b->tile_lo, b->tile_n, b->tQ, b->tS);
     batch_tile_scan<<<(b->F * 32 + 255) / 256, 256, 0, b->stream>>>(b->fp, b->fsum, b->cursor, b->ft_off, b->F,
-                                                                      b->tQ, b->tC, b->tT, b->fQu, b->fkeep,
+                                                                      b->tQ, b->tC, b->tT, b->tO, b->fsc, b->fQu, b->fkeep,
                                                                       b->flags);
-    batch_fill<<<b->T, TILE_THREADS, FILL_SMEM_BYTES, b->stream>>>(b->state[0], b->state[1], b->Ntot, b->fp, b->fsum, b->cursor,
-                                                     b->tile_f, b->tile_lo, b->tile_n, b->ft_off, b->tC, b->tT, b->fQu,
+    batch_fill<<<b->T, TILE_THREADS, 0, b->stream>>>(b->state[0], b->state[1], b->Ntot, b->fp, b->fsum, b->cursor,
+                                                     b->tile_f, b->tile_lo, b->tile_n, b->ft_off, b->tC, b->tT, b->tO, b->tS, b->fsc, b->fQu,
                                                      b->anc, b->flags);
     b->launches += 3;
     return cudaGetLastError();
@@ -681,7 +709,7 @@ void free_batch(ppf_batch *b)
     void *p[] = {b->fp, b->state[0], b->state[1], b->anc, b->Zp, b->unit_f, b->unit_lo, b->unit_n, b->fu_off,
                  b->upart, b->fsum, b->flags, b->fkeep, b->fsum_run, b->cursor, b->tile_f, b->tile_lo, b->tile_n,
                  b->ft_off,
-                 b->tQ, b->tC, b->tT, b->fQu};
+                 b->tQ, b->tC, b->tT, b->tO, b->tS, b->fsc, b->fQu};
     for (void *q : p)
         if (q)
             cudaFree(q);
@@ -796,9 +824,7 @@ ppf_status ppf_batch_create(const ppf_model *models, const int64_t *n, int32_t F
         cudaMemcpy(dv0A, v0A.data(), sizeof(float) * 2 * F, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(b->flags, 0, sizeof(int32_t)) != cudaSuccess ||
         cudaMemset(b->fkeep, 0, sizeof(int32_t) * F) != cudaSuccess || build_units(b, 1024) != cudaSuccess ||
-        build_tiles(b) != cudaSuccess ||
-        cudaFuncSetAttribute(batch_fill, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FILL_SMEM_BYTES) !=
-            cudaSuccess) {
+        build_tiles(b) != cudaSuccess) {
         cudaFree(dv0A);
         return fail(PPF_ECUDA);
     }

@@ -154,10 +154,11 @@ __device__ __forceinline__ void box_muller(float u1, float u2, float &z0, float 
 // ceil(log2 n) complement: s = 63 - ceil(log2 n), so that n * 2^s <= 2^63
 __host__ __device__ inline int scale_bits(int64_t n)
 {
-    int c = 0;
-    while (((int64_t)1 << c) < n)
-        ++c;
-    return 63 - c;
+#ifdef __CUDA_ARCH__
+    return n > 1 ? __clzll((long long)(n - 1)) - 1 : 63;
+#else
+    return n > 1 ? __builtin_clzll((unsigned long long)(n - 1)) - 1 : 63;
+#endif
 }
 
 // 2^f for f in [0, 1): Taylor polynomial of e^(f ln 2) to degree 9, the
@@ -178,28 +179,42 @@ __device__ __forceinline__ float exp2_frac(float f)
     return p;
 }
 
-// The integer part of the quantiser: q = floor(p 2^(s + kf)) for t > -64.
-__device__ __forceinline__ uint64_t quantise_tail(float t, float kf, float p, int s)
+// v >> n for any n (the PTX shift clamps n at 64, giving 0; the C++ operator
+// leaves n >= 64 undefined)
+__device__ __forceinline__ uint64_t shr_u64(uint64_t v, uint32_t n)
 {
-    const int e = s + (int)kf;
-    // p lies in [1, 2]: P = p 2^23 is its mantissa with the implicit bit,
-    // doubled when p = 2.  q = floor(P 2^(e - 23)) without branches:
-    // X = P 2^39 < 2^64, q = X / 2^(62 - e); e = 63 only for p = 1 (t = 0),
-    // and q = 0 for e < -1.
+    uint64_t r;
+    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+    return r;
+}
+
+// The quantiser's split of t = (lw - M) log2(e) <= 0 (clamped at -64 below:
+// smaller weights and NaN give q = 0): adding 1.5 2^23 with the sum rounded
+// down leaves floor(t) in the low mantissa bits, so the integer part costs an
+// addition instead of a round and a conversion (both run on the quarter-rate
+// conversion pipe).
+constexpr float FLOOR_MAGIC = 12582912.0f;              // 1.5 * 2^23
+constexpr uint32_t FLOOR_MAGIC_BITS = 0x4B400000u;
+
+// q = floor(p 2^(s + floor(t))), p in [1, 2], rb the bits of FLOOR_MAGIC +
+// floor(t): p's 24-bit mantissa sits at the top of 64 bits (its implicit bit
+// falls on the exponent's lowest bit, which is or-ed away) and is shifted
+// right by 63 - E, E = s + floor(t) + (p's exponent); E < 0 shifts everything out.
+__device__ __forceinline__ uint64_t quantise_tail(uint32_t rb, float p, int s)
+{
     const uint32_t pb = __float_as_uint(p);
-    const uint64_t X = ((uint64_t)((pb & 0x7FFFFFu) | 0x800000u) << (((pb >> 23) - 127u) & 1u)) << 39;
-    const int sh = 62 - e;
-    const uint64_t q = (sh < 0) ? (X << 1) : (X >> (sh < 63 ? sh : 63));
-    return (t > -64.0f && e >= -1) ? q : 0ull;  // t <= -64 or NaN: zero weight
+    const uint64_t X = (uint64_t)((pb << 8) | 0x80000000u) << 32;
+    const uint32_t n = (uint32_t)(63 + 127 - s) + FLOOR_MAGIC_BITS - rb - (pb >> 23);
+    return shr_u64(X, n);
 }
 
 __device__ __forceinline__ uint64_t quantise(float lw, float M, int s)
 {
     const float d = __fsub_rn(lw, M);
-    const float t = __fmul_rn(d, 0x1.715476p+0f);
-    const float kf = fmaxf(floorf(t), -64.0f);  // the clamp only affects results that are 0 anyway
-    const float f = __fsub_rn(t, kf);
-    return quantise_tail(t, kf, exp2_frac(f), s);
+    const float t = fmaxf(__fmul_rn(d, 0x1.715476p+0f), -64.0f);
+    const float r = __fadd_rd(t, FLOOR_MAGIC);
+    const float f = __fsub_rn(t, __fsub_rn(r, FLOOR_MAGIC));
+    return quantise_tail(__float_as_uint(r), exp2_frac(f), s);
 }
 
 // exp2_frac of two values at once: the same Horner steps as packed two-lane
@@ -225,13 +240,15 @@ __device__ __forceinline__ float2 exp2_frac2(float2 f)
 // scalar quantise bit for bit.
 __device__ __forceinline__ void quantise2(float a, float b, float M, int s, uint64_t &qa, uint64_t &qb)
 {
+    const float2 magic = make_float2(FLOOR_MAGIC, FLOOR_MAGIC);
     const float2 d = __fadd2_rn(make_float2(a, b), make_float2(-M, -M));
-    const float2 t = __fmul2_rn(d, make_float2(0x1.715476p+0f, 0x1.715476p+0f));
-    const float2 kf = make_float2(fmaxf(floorf(t.x), -64.0f), fmaxf(floorf(t.y), -64.0f));
-    const float2 f = __fadd2_rn(t, make_float2(-kf.x, -kf.y));
-    const float2 p = exp2_frac2(f);
-    qa = quantise_tail(t.x, kf.x, p.x, s);
-    qb = quantise_tail(t.y, kf.y, p.y, s);
+    float2 t = __fmul2_rn(d, make_float2(0x1.715476p+0f, 0x1.715476p+0f));
+    t = make_float2(fmaxf(t.x, -64.0f), fmaxf(t.y, -64.0f));
+    const float2 r = __fadd2_rd(t, magic);
+    const float2 nk = __ffma2_rn(r, make_float2(-1.0f, -1.0f), magic);  // -floor(t), exact
+    const float2 p = exp2_frac2(__fadd2_rn(t, nk));
+    qa = quantise_tail(__float_as_uint(r.x), p.x, s);
+    qb = quantise_tail(__float_as_uint(r.y), p.y, s);
 }
 
 // Number of systematic tickets below cumulative weight c (the per-group

@@ -22,7 +22,7 @@ struct NvtxRange {
 constexpr int TILE = 4096;          // particles per resampling tile (256 threads x 16)
 constexpr int TILE_THREADS = 256;
 constexpr int TILE_ITEMS = TILE / TILE_THREADS;
-constexpr int ITEM_TICKETS = 8192;  // tickets per fill work item
+constexpr int ITEM_TICKETS = 8184;  // tickets per fill work item (below 2^13: the ticket counts' fixed point)
 constexpr int COPY_CHUNK = 8192;    // slots per routing-copy work item
 constexpr int MAX_RADIUS = 8;
 constexpr int MAX_SCHED_GROUPS = 16384;
@@ -72,7 +72,8 @@ struct DevSummary {
     uint64_t Q, u;             // last global resample: total fixed-point weight, offset
     uint64_t qN;               // and Q = qN N + qR (the ticket spacing in whole and remainder)
     uint32_t qR;
-    int32_t n_items;           // fill work items of the last resample
+    uint32_t tsv;              // N / Q for the fill's ticket counts (TicketScale)
+    int32_t tsr, tsl;
     int32_t n_chunks;          // routing-copy work items of the last RPA resample
     int64_t mig;               // RNA: slots migrating to the next group
     int32_t involved;          // ARNA: groups that proportional allocation gives at least their size
@@ -92,7 +93,7 @@ struct DevSummary {
 };
 
 // two-stage RPA: one group's own systematic draw and where its offspring go
-// (see group_grid_kernel), read by the group's block as six 16-byte loads
+// (see group_grid_kernel), read by the group's block as seven 16-byte loads
 struct alignas(16) GroupGrid {
     uint64_t Ca;     // cumulative fixed-point weight below the group
     uint64_t Q;      // the group's total
@@ -105,13 +106,17 @@ struct alignas(16) GroupGrid {
     int64_t shift;   // the slot of its first kept offspring (the balanced offset)
     uint32_t qR;
     uint32_t nt;     // its offspring count (0: nothing to draw)
+    uint32_t tsv;    // nt / Q for the ticket counts (TicketScale)
+    int32_t tsr, tsl;
+    int32_t off;     // run_offset of its first ticket
 };
 
 struct Scratch {
     uint64_t *Qt;      // [T]   tile totals
+    uint64_t *St;      // [8T]  per tile: the weight below each of its 8 strips of 512 particles
     uint64_t *Ct;      // [T+1] exclusive tile prefix
     int64_t *Tt;       // [T+1] tickets below each tile start
-    int32_t *item_off; // [T+1] fill work-item prefix per tile
+    int32_t *To;       // [T]   run_offset of each tile's tickets (the fill's ticket counts)
     int32_t *extra;    // [2 (N / ITEM_TICKETS + 1)] the fill's further runs (tile, run) of ticket-heavy tiles
     uint64_t *Cbl;     // [G+1] local prefix at group starts (within their tile)
     int64_t *Tg;       // [G+1] tickets below each group start
@@ -134,6 +139,7 @@ struct ppf_ctx {
     ppf_model m;
     int64_t N;
     int32_t group_size, G, T;     // groups, resampling tiles
+    bool uneven;                  // the groups may differ from the balanced layout (LGS, ppf_set_groups)
     cudaStream_t stream;
     cudaStream_t side_stream;     // the RPA schedule, concurrent with the fill
     cudaEvent_t ev_scan, ev_sched;  // fork after the tile scan, join before the routing copy
@@ -220,6 +226,9 @@ cudaError_t resample_kernel_attributes();
 cudaError_t launch_resample_global(ppf_ctx *c, int scheme, double ess_thr);
 cudaError_t launch_resample_rna(ppf_ctx *c, float alpha, double ess_thr);
 cudaError_t launch_resample_arna(ppf_ctx *c, float alpha, double ess_thr);
+cudaError_t launch_fill_plain(const float *lw, int64_t N, int32_t T, const DevSummary *sum, const uint64_t *Ct,
+                              const int64_t *Tt, const int32_t *To, const uint64_t *St, const int2 *extra,
+                              int32_t *out, cudaStream_t stream);
 cudaError_t launch_identity(ppf_ctx *c, int32_t *dst);
 cudaError_t launch_pending(ppf_ctx *c, int32_t *anc_out, float *lwp_out);
 cudaError_t launch_fill_f32(ppf_ctx *c, float *dst, float v);

@@ -29,18 +29,14 @@ namespace ppf {
 // kernels of ppf_resample.cu used unchanged
 __global__ void __launch_bounds__(TILE_THREADS, 5) tile_totals_kernel(const float *__restrict__ lw, int64_t N,
                                                                       const DevSummary *__restrict__ sum,
-                                                                      double ess_thr, uint64_t *__restrict__ Qt);
+                                                                      double ess_thr, uint64_t *__restrict__ Qt,
+                                                                      uint64_t *__restrict__ St);
 __global__ void __launch_bounds__(1024) tile_scan_kernel(int64_t N, int32_t T, const uint64_t *__restrict__ Qt, uint64_t *__restrict__ Ct,
-                                 int64_t *__restrict__ Tt, int32_t *__restrict__ item_off,
-                                 int32_t *__restrict__ item_tile, DevSummary *sum, double ess_thr, uint64_t seed,
+                                 int64_t *__restrict__ Tt, DevSummary *sum, double ess_thr, uint64_t seed,
                                  uint32_t fid, uint32_t frame, const int64_t *__restrict__ goff, int32_t G, int rpa,
                                  const uint64_t *__restrict__ Cbl, int64_t *__restrict__ Tg, int32_t smem_tiles,
-                                 Divisor ndiv, int prefix_only, int2 *__restrict__ extra);
-__global__ void __launch_bounds__(TILE_THREADS) fill_kernel(const float *__restrict__ lw, int64_t N, int32_t T, Divisor ndiv,
-                            const DevSummary *__restrict__ sum, const uint64_t *__restrict__ Ct,
-                            const int64_t *__restrict__ Tt, const int32_t *__restrict__ item_off,
-                            const int32_t *__restrict__ item_tile, int32_t *__restrict__ out);
-
+                                 Divisor ndiv, int prefix_only, int2 *__restrict__ extra,
+                                 int32_t *__restrict__ To);
 namespace {
 
 constexpr int64_t NOALLOC_MAX_N = (int64_t)1 << 24;               // particles per call
@@ -53,8 +49,10 @@ constexpr size_t OFF_MAX = align256(OFF_SUM + sizeof(DevSummary));   // ordered 
 constexpr size_t OFF_QT = align256(OFF_MAX + 2 * sizeof(uint32_t));
 constexpr size_t OFF_CT = align256(OFF_QT + sizeof(uint64_t) * NOALLOC_MAX_T);
 constexpr size_t OFF_TT = align256(OFF_CT + sizeof(uint64_t) * (NOALLOC_MAX_T + 1));
-constexpr size_t OFF_IT = align256(OFF_TT + sizeof(int64_t) * (NOALLOC_MAX_T + 1));
-constexpr size_t SCRATCH_BYTES = align256(OFF_IT + sizeof(int32_t) * (NOALLOC_MAX_T + 1));  // ~113 KB
+constexpr size_t OFF_EX = align256(OFF_TT + sizeof(int64_t) * (NOALLOC_MAX_T + 1));  // further runs (int2)
+constexpr size_t OFF_TO = align256(OFF_EX + sizeof(int2) * (NOALLOC_MAX_N / ITEM_TICKETS + 1));
+constexpr size_t OFF_ST = align256(OFF_TO + sizeof(int32_t) * NOALLOC_MAX_T);
+constexpr size_t SCRATCH_BYTES = align256(OFF_ST + sizeof(uint64_t) * STRIPS * NOALLOC_MAX_T);  // ~391 KB
 
 static __device__ __align__(256) unsigned char g_scratch[SCRATCH_BYTES];
 
@@ -170,7 +168,7 @@ unsigned char *scratch_address(int dev, cudaError_t *err)
         *err = cudaGetSymbolAddress(&p, g_scratch);
         if (*err != cudaSuccess)
             return nullptr;
-        // the fill kernel's dynamic shared memory size (an attribute, no allocation)
+        // the kernels' dynamic shared memory sizes (attributes, no allocation)
         *err = resample_kernel_attributes();
         if (*err != cudaSuccess)
             return nullptr;
@@ -203,22 +201,22 @@ extern "C" ppf_status ppf_systematic_resample_noalloc(const float *lw_dev, int64
     uint64_t *Qt = reinterpret_cast<uint64_t *>(s + OFF_QT);
     uint64_t *Ct = reinterpret_cast<uint64_t *>(s + OFF_CT);
     int64_t *Tt = reinterpret_cast<int64_t *>(s + OFF_TT);
-    int32_t *item_off = reinterpret_cast<int32_t *>(s + OFF_IT);
+    int2 *extra = reinterpret_cast<int2 *>(s + OFF_EX);
+    int32_t *To = reinterpret_cast<int32_t *>(s + OFF_TO);
+    uint64_t *St = reinterpret_cast<uint64_t *>(s + OFF_ST);
     const int32_t T = (int32_t)((n + TILE - 1) / TILE);
     noalloc_clear_kernel<<<1, 32, 0, st>>>(s);
     const int gmax = (int)((n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024);
     noalloc_max_kernel<<<gmax, 256, 0, st>>>(lw_dev, n, s);
     // (every call resamples: the N_eff threshold is +inf)
-    tile_totals_kernel<<<T, TILE_THREADS, 0, st>>>(lw_dev, n, sum, INFINITY, Qt);
-    // (no item-to-tile map: the fill blocks find their tile by binary search)
+    tile_totals_kernel<<<T, TILE_THREADS, 0, st>>>(lw_dev, n, sum, INFINITY, Qt, St);
     // (T <= 4096 tiles: the scan's tile values, 32 KB, fit the default shared memory)
-    tile_scan_kernel<<<1, 1024, sizeof(uint64_t) * (T + 1), st>>>(n, T, Qt, Ct, Tt, item_off, nullptr, sum, INFINITY,
+    tile_scan_kernel<<<1, 1024, sizeof(uint64_t) * (T + 1), st>>>(n, T, Qt, Ct, Tt, sum, INFINITY,
                                                                   seed, filter_id, (uint32_t)frame, nullptr, 0, 0,
                                                                   nullptr, nullptr, T, make_divisor((uint32_t)n), 0,
-                                                                  nullptr);
-    const int max_items = T + (int)((n + ITEM_TICKETS - 1) / ITEM_TICKETS);
-    fill_kernel<<<max_items, TILE_THREADS, FILL_SMEM_BYTES, st>>>(lw_dev, n, T, make_divisor((uint32_t)n), sum, Ct,
-                                                                  Tt, item_off, nullptr, anc_dev);
+                                                                  extra, To);
+    if (launch_fill_plain(lw_dev, n, T, sum, Ct, Tt, To, St, extra, anc_dev, st) != cudaSuccess)
+        return PPF_ECUDA;
     noalloc_identity_if_degenerate<<<gmax, 256, 0, st>>>(anc_dev, n, s);
     return cudaGetLastError() == cudaSuccess ? PPF_OK : PPF_ECUDA;
 }

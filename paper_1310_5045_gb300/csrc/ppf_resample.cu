@@ -53,75 +53,81 @@ __device__ __forceinline__ int64_t balanced_offset(const Balanced &b, int32_t g)
 }
 
 // ---------------------------------------------------------------- R1 tiles
-// Tile totals Q_t: every thread loads its four float4 (coalesced, all in
-// flight together), then quantises them two at a time; one block sum.  No
-// shared buffer, so more blocks fit an SM.
+// Tile totals Q_t and the prefix of every tile's strips: every warp loads its
+// strip (coalesced, all 16 values in flight together) and quantises them two
+// at a time; the warp sums meet in shared memory.  Integer sums: any order.
+// 33 us at 38M particles (48 before the quantiser's floor by a rounded-down
+// addition), 22 us at the copy bandwidth.
 __global__ void __launch_bounds__(TILE_THREADS, 5) tile_totals_kernel(const float *__restrict__ lw, int64_t N,
                                                                       const DevSummary *__restrict__ sum,
-                                                                      double ess_thr, uint64_t *__restrict__ Qt)
+                                                                      double ess_thr, uint64_t *__restrict__ Qt,
+                                                                      uint64_t *__restrict__ St)
 {
     // Blocks take tiles blockIdx.x, + gridDim.x, ... (one each when the grid
     // has a block per tile).  A full, aligned tile's loads go out one tile
     // ahead, so that they are in flight while the block quantises the tile
-    // before and waits at its reduction.
+    // before and waits at its reduction; any other tile is loaded when it is
+    // its turn.
     if (kept_by_ess(sum, ess_thr))
         return;
-    constexpr int V = TILE / 4 / TILE_THREADS;
-    __shared__ uint64_t wsum[TILE_THREADS / 32];
-    const int64_t T = (N + TILE - 1) / TILE;
+    __shared__ uint64_t wsum[2][STRIPS];
+    const int32_t T = (int32_t)((N + TILE - 1) / TILE);
+    const int32_t T_full = (reinterpret_cast<uintptr_t>(lw) & 15) == 0 ? (int32_t)(N / TILE) : 0;
     const float M = sum->M;
     const int s = scale_bits(N);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    auto full_tile = [&](int64_t t) {
-        const int64_t lo = t * TILE;
-        return N - lo >= TILE && ((reinterpret_cast<uintptr_t>(lw + lo) & 15) == 0);
-    };
-    auto load = [&](int64_t t, float4 (&v)[V]) {
-        const float4 *v4 = reinterpret_cast<const float4 *>(lw + t * TILE) + threadIdx.x;
+    const float4 *v4 = reinterpret_cast<const float4 *>(lw) + warp * (TILE / STRIPS / 4) + lane;
+    auto load = [&](int32_t t, float (&v)[TILE_ITEMS]) {
 #pragma unroll
-        for (int k = 0; k < V; ++k)
-            v[k] = __ldg(v4 + k * TILE_THREADS);
+        for (int k = 0; k < TILE_ITEMS / 4; ++k) {
+            const float4 x = __ldg(v4 + (int64_t)t * (TILE / 4) + 32 * k);
+            v[4 * k] = x.x; v[4 * k + 1] = x.y; v[4 * k + 2] = x.z; v[4 * k + 3] = x.w;
+        }
     };
-    int64_t t = blockIdx.x;
-    float4 v[V];
-    if (t < T && full_tile(t))
-        load(t, v);
-    for (; t < T; t += gridDim.x) {
-        const int64_t tn = t + gridDim.x;
-        float4 vn[V];
-        if (tn < T && full_tile(tn))
-            load(tn, vn);
+    int buf = 0;
+    auto finish = [&](int32_t t, const float (&v)[TILE_ITEMS]) {
         uint64_t acc = 0;
-        if (full_tile(t)) {
 #pragma unroll
-            for (int k = 0; k < V; ++k) {
-                uint64_t a, b, c, d;
-                quantise2(v[k].x, v[k].y, M, s, a, b);
-                quantise2(v[k].z, v[k].w, M, s, c, d);
-                acc += a + b + c + d;
-            }
-        } else {
-            const int64_t lo = t * TILE;
-            const int n = (int)(N - lo < TILE ? N - lo : TILE);
-            for (int e = threadIdx.x; e < n; e += blockDim.x)
-                acc += quantise(__ldg(lw + lo + e), M, s);
+        for (int k = 0; k < TILE_ITEMS; k += 2) {
+            uint64_t a, b;
+            quantise2(v[k], v[k + 1], M, s, a, b);
+            acc += a + b;
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1)
             acc += __shfl_xor_sync(0xffffffffu, acc, o);
         if (lane == 0)
-            wsum[warp] = acc;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            uint64_t total = 0;
-            for (int w = 0; w < TILE_THREADS / 32; ++w)
-                total += wsum[w];
-            Qt[t] = total;
+            wsum[buf][warp] = acc;
+        __syncthreads();  // (two buffers: the next tile's sums never meet this one's readers)
+        if (threadIdx.x <= STRIPS) {
+            uint64_t below = 0;
+            for (int w = 0; w < (int)threadIdx.x; ++w)
+                below += wsum[buf][w];
+            if (threadIdx.x < STRIPS)
+                St[(int64_t)t * STRIPS + threadIdx.x] = below;
+            else
+                Qt[t] = below;
         }
-        __syncthreads();  // wsum is rewritten for the next tile
+        buf ^= 1;
+    };
+    int32_t t = blockIdx.x;
+    float v[TILE_ITEMS];
+    if (t < T_full)
+        load(t, v);
+    for (; t < T_full; t += (int32_t)gridDim.x) {
+        const int32_t tn = t + (int32_t)gridDim.x;
+        float vn[TILE_ITEMS];
+        if (tn < T_full)
+            load(tn, vn);
+        finish(t, v);
 #pragma unroll
-        for (int k = 0; k < V; ++k)
+        for (int k = 0; k < TILE_ITEMS; ++k)
             v[k] = vn[k];
+    }
+    for (; t < T; t += (int32_t)gridDim.x) {
+        const int64_t lo = (int64_t)t * TILE;
+        strip_load(lw + lo, (int)(N - lo < TILE ? N - lo : TILE), v);
+        finish(t, v);
     }
 }
 
@@ -137,14 +143,15 @@ constexpr int GT_MASKED = 4;  // group starts per tile handled by masked sums
 
 // The thread's part of the tile total (acc[GT_MASKED]) and of the prefix
 // before each of the NS group starts at local positions spos[j] (acc[j]).
-// Thread t holds the quads 4 (t + k TILE_THREADS) .. + 3: a quad lies wholly
-// below or above a start except the one quad that holds it, so each start
-// costs a select of the quad's sum, and the partial quad a few more.
+// A thread holds the quads of its warp's strip that strip_load gives it: a
+// quad lies wholly below or above a start except the one quad that holds it,
+// so each start costs a select of the quad's sum, and the partial quad a few more.
 template <int NS>
-__device__ __forceinline__ void masked_sums(const float4 (&v)[TILE / 4 / TILE_THREADS], const int32_t *spos, float M,
-                                            int s, uint64_t (&acc)[GT_MASKED + 1])
+__device__ __forceinline__ void masked_sums(const float (&v)[TILE_ITEMS], const int32_t *spos, float M, int s,
+                                            uint64_t (&acc)[GT_MASKED + 1])
 {
-    constexpr int V = TILE / 4 / TILE_THREADS;
+    constexpr int V = TILE_ITEMS / 4;
+    const int q0 = (int)(threadIdx.x >> 5) * (TILE / STRIPS) + 4 * (int)(threadIdx.x & 31);
     int p[NS > 0 ? NS : 1];
 #pragma unroll
     for (int j = 0; j < NS; ++j)
@@ -155,11 +162,11 @@ __device__ __forceinline__ void masked_sums(const float4 (&v)[TILE / 4 / TILE_TH
 #pragma unroll
     for (int k = 0; k < V; ++k) {
         uint64_t w0, w1, w2, w3;
-        quantise2(v[k].x, v[k].y, M, s, w0, w1);
-        quantise2(v[k].z, v[k].w, M, s, w2, w3);
+        quantise2(v[4 * k], v[4 * k + 1], M, s, w0, w1);
+        quantise2(v[4 * k + 2], v[4 * k + 3], M, s, w2, w3);
         const uint64_t w01 = w0 + w1, qs = w01 + w2 + w3;
         acc[GT_MASKED] += qs;
-        const int e0 = 4 * ((int)threadIdx.x + k * TILE_THREADS);
+        const int e0 = q0 + 128 * k;
 #pragma unroll
         for (int j = 0; j < NS; ++j) {
             const int d = p[j] - e0;  // elements of the quad below start j
@@ -171,30 +178,24 @@ __device__ __forceinline__ void masked_sums(const float4 (&v)[TILE / 4 / TILE_TH
 
 __global__ void __launch_bounds__(TILE_THREADS, 5) tile_group_totals_kernel(
     const float *__restrict__ lw, int64_t N, const DevSummary *__restrict__ sum, double ess_thr,
-    uint64_t *__restrict__ Qt, const int64_t *__restrict__ goff, int32_t G, uint64_t *__restrict__ Cbl,
-    int32_t *__restrict__ tile_g)
+    uint64_t *__restrict__ Qt, uint64_t *__restrict__ St, const int64_t *__restrict__ goff, int32_t G,
+    uint64_t *__restrict__ Cbl, int32_t *__restrict__ tile_g)
 {
     if (kept_by_ess(sum, ess_thr))
         return;
-    __shared__ uint64_t buf[TILE_SMEM_U64];
-    __shared__ uint64_t red[33];
+    __shared__ uint64_t sums[TILE];  // the tile's inclusive sums (only for tiles with many group starts)
+    __shared__ uint64_t red[STRIPS];
     __shared__ int32_t gfirst, nstart;
     __shared__ int32_t spos[GT_MASKED];
-    __shared__ uint64_t wsum[TILE_THREADS / 32][GT_MASKED + 1];
+    __shared__ uint64_t wsum[STRIPS][GT_MASKED], stot[STRIPS];
     const int64_t lo = (int64_t)blockIdx.x * TILE;
     const int n = (int)(N - lo < TILE ? N - lo : TILE);
     // the weights first, so that their loads are in flight during the search
-    // warp 0 does for the tile's group starts.  Thread t holds elements
-    // 4 (t + k TILE_THREADS) + j, j < 4.
-    constexpr int V = TILE / 4 / TILE_THREADS;
+    // warp 0 does for the tile's group starts
     const bool full = n == TILE && ((reinterpret_cast<uintptr_t>(lw + lo) & 15) == 0);
-    float4 v[V];
-    if (full) {
-        const float4 *v4 = reinterpret_cast<const float4 *>(lw + lo) + threadIdx.x;
-#pragma unroll
-        for (int k = 0; k < V; ++k)
-            v[k] = __ldg(v4 + k * TILE_THREADS);
-    }
+    float v[TILE_ITEMS];
+    if (full)
+        strip_load(lw + lo, n, v);
     if (threadIdx.x < 32) {
         // warp 0: the first g with goff[g] >= lo (goff[G] = N >= lo, so it
         // exists).  The first round probes the 32 groups around the balanced
@@ -269,46 +270,57 @@ __global__ void __launch_bounds__(TILE_THREADS, 5) tile_group_totals_kernel(
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1)
                     x += __shfl_xor_sync(0xffffffffu, x, o);
-                if (lane == 0)
-                    wsum[warp][j] = x;
+                if (lane == 0) {
+                    if (j == GT_MASKED)
+                        stot[warp] = x;
+                    else
+                        wsum[warp][j] = x;
+                }
             }
         }
         __syncthreads();
-        if (threadIdx.x <= GT_MASKED) {
+        store_strips(stot, St + (int64_t)blockIdx.x * STRIPS, Qt + blockIdx.x);
+        if (threadIdx.x >= 32 && threadIdx.x < 32 + ns) {
             uint64_t x = 0;
-            if (threadIdx.x < ns || threadIdx.x == GT_MASKED)
-                for (int w = 0; w < TILE_THREADS / 32; ++w)
-                    x += wsum[w][threadIdx.x];
-            if (threadIdx.x == GT_MASKED)
-                Qt[blockIdx.x] = x;
-            else if (threadIdx.x < ns)
-                Cbl[gfirst + threadIdx.x] = x;
+            for (int w = 0; w < STRIPS; ++w)
+                x += wsum[w][threadIdx.x - 32];
+            Cbl[gfirst + threadIdx.x - 32] = x;
         }
         return;
     }
-    uint64_t q[TILE_ITEMS];
-    tile_weights(lw, lo, n, M, s, buf, q);
-    const uint64_t total = tile_scan(q, buf, red);
-    if (threadIdx.x == 0)
-        Qt[blockIdx.x] = total;
+    float w[TILE_ITEMS];
+    tile_load16(lw, N, lo, n, w);
+    __shared__ uint64_t bred[33];
+    uint64_t btot;
+    TileSums ts;
+    tile_quantise(w, M, s, ts);
+    const uint64_t pre = block_excl_scan_u64(ts.loc[TILE_ITEMS - 1], bred, &btot);
+#pragma unroll
+    for (int k = 0; k < TILE_ITEMS; ++k)
+        sums[threadIdx.x * TILE_ITEMS + k] = pre + ts.loc[k];
+    __syncthreads();
+    if (threadIdx.x < STRIPS)
+        red[threadIdx.x] = sums[TILE / STRIPS * (threadIdx.x + 1) - 1] -
+                           (threadIdx.x ? sums[TILE / STRIPS * threadIdx.x - 1] : 0ull);
+    __syncwarp();
+    store_strips(red, St + (int64_t)blockIdx.x * STRIPS, Qt + blockIdx.x);
     __syncthreads();
     for (int32_t g = gfirst + threadIdx.x; g <= G; g += blockDim.x) {
         const int64_t pos = goff[g];
         if (pos >= lo + n)
             break;
         const int k = (int)(pos - lo);
-        Cbl[g] = (k == 0) ? 0ull : buf[padc(k - 1)];
+        Cbl[g] = (k == 0) ? 0ull : sums[k - 1];
     }
 }
 
 // ---------------------------------------------------------------- R2 scan
 // One block: exclusive tile prefix, total Q, ticket offset u, tickets below
-// each tile start, fill work items (and the tile of each item when item_tile
-// is given); for RPA (rpa = 1) and ARNA (rpa = 2) the tickets below each
-// group start.  A proportional draw (rpa != 2) at a low N_eff also sets the
-// next step to the direct likelihood path.  With prefix_only the kernel stops
-// after the prefix and the draw (tile_tickets_kernel does the rest in
-// parallel).
+// each tile start and the list of the fill's further runs; for RPA (rpa = 1)
+// and ARNA (rpa = 2) the tickets below each group start.  A proportional draw
+// (rpa != 2) at a low N_eff also sets the next step to the direct likelihood
+// path.  With prefix_only the kernel stops after the prefix and the draw
+// (tile_tickets_kernel does the rest in parallel).
 // When the T + 1 tile values fit the dynamic shared memory (T <= smem_tiles),
 // they are loaded there with coalesced reads, and each of the two prefix sums
 // gives every thread one contiguous segment: a local sum, one block scan,
@@ -316,15 +328,16 @@ __global__ void __launch_bounds__(TILE_THREADS, 5) tile_group_totals_kernel(
 // blockDim consecutive entries, each round closed by a block scan.
 __global__ void __launch_bounds__(1024) tile_scan_kernel(
     int64_t N, int32_t T, const uint64_t *__restrict__ Qt, uint64_t *__restrict__ Ct, int64_t *__restrict__ Tt,
-    int32_t *__restrict__ item_off, int32_t *__restrict__ item_tile, DevSummary *sum, double ess_thr, uint64_t seed,
+    DevSummary *sum, double ess_thr, uint64_t seed,
     uint32_t fid, uint32_t frame, const int64_t *__restrict__ goff, int32_t G, int rpa,
     const uint64_t *__restrict__ Cbl, int64_t *__restrict__ Tg, int32_t smem_tiles, Divisor ndiv, int prefix_only,
-    int2 *__restrict__ extra)
+    int2 *__restrict__ extra, int32_t *__restrict__ To)
 {
     extern __shared__ uint64_t sT[];  // (smem_tiles + 1) tile values
     __shared__ uint64_t red[33];
     __shared__ uint64_t su, s_qN;
     __shared__ uint32_t s_qR;
+    __shared__ TicketScale s_sc;
     if (threadIdx.x == 0) {
         sum->n_split = 0;  // the two-stage draw's split list is rebuilt after the scan
         sum->n_runs = 0;
@@ -334,7 +347,6 @@ __global__ void __launch_bounds__(1024) tile_scan_kernel(
         if (threadIdx.x == 0) {
             sum->degenerate = 1;
             sum->flags |= FLAG_KEPT;
-            sum->n_items = 0;
             sum->links = 0;
             sum->moved = 0;
         }
@@ -382,84 +394,50 @@ __global__ void __launch_bounds__(1024) tile_scan_kernel(
         s_qR = (uint32_t)(total % (uint64_t)N);
         sum->qN = s_qN;
         sum->qR = s_qR;
+        if (!deg) {
+            const TicketScale sc = ticket_scale(total, (uint32_t)N);
+            sum->tsv = sc.v;
+            sum->tsr = sc.sr;
+            sum->tsl = sc.sl;
+            s_sc = sc;
+        }
         su = deg ? 0ull : ticket_offset(seed, fid, frame, PURPOSE_RESAMPLE, 0u, total);
         sum->u = su;
     }
     __syncthreads();
     const uint64_t Q = total, u = su;
     const TicketGrid tg = ticket_grid(Q, u, s_qN, s_qR, ndiv);
-    if (Q == 0ull) {
-        if (threadIdx.x == 0)
-            sum->n_items = 0;
+    if (Q == 0ull)
         return;
-    }
     if (threadIdx.x == 0 && rpa != 2 && sum->ess < (double)N / BIN_CONCENTRATE)
         sum->bin_next = 0;  // a concentrating proportional draw: the next step is direct
     if (prefix_only) {  // tile_tickets_kernel takes it from here, one thread per tile and group
-        if (threadIdx.x == 0) {
-            sum->n_items = 0;
-            if (!rpa) {
-                sum->links = 0;
-                sum->moved = 0;
-            }
+        if (threadIdx.x == 0 && !rpa) {
+            sum->links = 0;
+            sum->moved = 0;
         }
         return;
     }
     for (int t = threadIdx.x; t <= T; t += blockDim.x) {
-        const int64_t v = (t == T) ? N : tickets_below_grid(in_smem ? sT[t] : Ct[t], tg);
+        const uint64_t c = in_smem ? sT[t] : Ct[t];
+        const int64_t v = (t == T) ? N : tickets_below_grid(c, tg);
         Tt[t] = v;
+        if (t < T)
+            To[t] = run_offset(c, tg, s_sc, v, true);
         if (in_smem)
             sT[t] = (uint64_t)v;  // each thread rewrites only the entries it read
     }
     __syncthreads();
-    if (extra) {  // the tile-major fill's further runs of ticket-heavy tiles, as tile_tickets_kernel lists them
-        for (int t = threadIdx.x; t < T; t += blockDim.x) {
-            const int64_t a = in_smem ? (int64_t)sT[t] : Tt[t], b = in_smem ? (int64_t)sT[t + 1] : Tt[t + 1];
-            const int64_t runs = (b - a + ITEM_TICKETS - 1) / ITEM_TICKETS;
-            if (runs > 1) {
-                const int32_t pos = atomicAdd(&sum->n_extra, (int32_t)(runs - 1));
-                for (int64_t k = 1; k < runs; ++k)
-                    extra[pos + k - 1] = make_int2(t, (int32_t)k);
-            }
+    // the fill's further runs of ticket-heavy tiles, as tile_tickets_kernel lists them
+    for (int t = threadIdx.x; t < T; t += blockDim.x) {
+        const int64_t a = in_smem ? (int64_t)sT[t] : Tt[t];
+        const int64_t b = (t + 1 == T) ? N : (in_smem ? (int64_t)sT[t + 1] : Tt[t + 1]);
+        const int64_t runs = (b - a + ITEM_TICKETS - 1) / ITEM_TICKETS;
+        if (runs > 1) {
+            const int32_t pos = atomicAdd(&sum->n_extra, (int32_t)(runs - 1));
+            for (int64_t k = 1; k < runs; ++k)
+                extra[pos + k - 1] = make_int2(t, (int32_t)k);
         }
-    }
-    // fill work items: ceil(tickets / ITEM_TICKETS) per tile
-    uint64_t items_total = 0;
-    if (in_smem) {
-        auto items_of = [&](int t) -> int32_t {
-            return (int32_t)(((int64_t)sT[t + 1] - (int64_t)sT[t] + ITEM_TICKETS - 1) / ITEM_TICKETS);
-        };
-        uint64_t loc = 0;
-        for (int t = s0; t < s1; ++t)
-            loc += (uint64_t)items_of(t);
-        int32_t off = (int32_t)block_excl_scan_u64(loc, red, &items_total);
-        for (int t = s0; t < s1; ++t) {
-            const int32_t cnt = items_of(t);
-            item_off[t] = off;
-            if (item_tile)
-                for (int32_t k = 0; k < cnt; ++k)
-                    item_tile[off + k] = t;
-            off += cnt;
-        }
-    } else {
-        for (int base = 0; base < T; base += blockDim.x) {
-            const int t = base + threadIdx.x;
-            const uint64_t cnt =
-                (t < T) ? (uint64_t)((Tt[t + 1] - Tt[t] + ITEM_TICKETS - 1) / ITEM_TICKETS) : 0ull;
-            uint64_t tot;
-            const uint64_t ex = block_excl_scan_u64(cnt, red, &tot);
-            if (t < T) {
-                item_off[t] = (int32_t)(items_total + ex);
-                if (item_tile)
-                    for (uint64_t k = 0; k < cnt; ++k)
-                        item_tile[items_total + ex + k] = t;
-            }
-            items_total += tot;
-        }
-    }
-    if (threadIdx.x == 0) {
-        item_off[T] = (int32_t)items_total;
-        sum->n_items = (int32_t)items_total;
     }
     if (rpa) {
         for (int g = threadIdx.x; g <= G; g += blockDim.x) {
@@ -485,7 +463,7 @@ __global__ void __launch_bounds__(1024) tile_scan_kernel(
 __global__ void __launch_bounds__(256) tile_tickets_kernel(
     int64_t N, int32_t T, const uint64_t *__restrict__ Ct, int64_t *__restrict__ Tt, DevSummary *__restrict__ sum,
     Divisor ndiv, const int64_t *__restrict__ goff, int32_t G, int rpa, const uint64_t *__restrict__ Cbl,
-    int64_t *__restrict__ Tg, int2 *__restrict__ extra)
+    int64_t *__restrict__ Tg, int2 *__restrict__ extra, int32_t *__restrict__ To)
 {
     if (sum->degenerate)
         return;  // kept by the N_eff test, or no usable weight
@@ -495,6 +473,7 @@ __global__ void __launch_bounds__(256) tile_tickets_kernel(
         const int64_t a = (i == T) ? N : tickets_below_grid(Ct[i], tg);
         Tt[i] = a;
         if (i < T) {
+            To[i] = run_offset(Ct[i], tg, TicketScale{sum->tsv, sum->tsr, sum->tsl}, a, true);
             const int64_t b = (i + 1 == T) ? N : tickets_below_grid(Ct[i + 1], tg);
             const int64_t runs = (b - a + ITEM_TICKETS - 1) / ITEM_TICKETS;
             if (runs > 1) {
@@ -527,75 +506,80 @@ struct KeptTable {
     int64_t shift[KT_GROUPS];      // a kept ticket j goes to slot j + shift
 };
 
-// ticket_parents_contig with the kept / sent split: per staged chunk, every
-// group's kept piece goes to anc (shifted to its balanced slot) and its sent
-// piece to anc_sys + sent_shift, each as one store_staged run.  With kt.n < 0
+// The kept / sent split of the parents of tickets [c, c + m): every group's
+// kept piece goes to anc (shifted to its balanced slot) and its sent piece to
+// anc_sys + sent_shift, each as one store_staged run.  With kt.n < 0
 // every ticket finds its group among Tg[0..G] by bisection (a tile crossed by
 // more than KT_GROUPS groups).
-__device__ __forceinline__ void ticket_parents_routed(const uint64_t *C, int n, uint64_t c0, const TicketGrid &tg,
-                                                      int64_t j_lo, int64_t j_hi, uint16_t *stage,
-                                                      const KeptTable &kt, int32_t *__restrict__ anc,
-                                                      int32_t *__restrict__ anc_sys, int64_t sent_shift,
-                                                      int32_t base, int64_t N, int32_t G, const Balanced &bl,
-                                                      const int64_t *__restrict__ Tg, const int32_t *flags)
-{
-    for (int64_t c = j_lo; c < j_hi; c += STAGE_TICKETS) {
-        const int64_t ce = (j_hi - c < STAGE_TICKETS) ? j_hi : c + STAGE_TICKETS;
-        const int m = (int)(ce - c);
-        ticket_parents(C, n, c0, tg, c, m, [&](int64_t j, int i) { stage[j - c] = (uint16_t)i; });
-        __syncthreads();
+struct EmitRouted {
+    static constexpr bool DIRECT = false;
+    const KeptTable &kt;
+    int32_t *__restrict__ anc;
+    int32_t *__restrict__ anc_sys;
+    int64_t sent_shift;
+    int32_t base;
+    int n;
+    int64_t N;
+    int32_t G;
+    const Balanced &bl;
+    const int64_t *__restrict__ Tg;
+    const int32_t *flags;
+    __device__ __forceinline__ int lead(int64_t) const { return 0; }
+    __device__ __forceinline__ void piece(int32_t *dst, int64_t slot, const uint16_t *st, int m) const
+    {
+        if (slot >= 0 && slot + m <= N)
+            store_staged(dst + slot, st, m, base, n, flags);
+        else if (threadIdx.x == 0)
+            atomicOr(const_cast<int32_t *>(flags), FLAG_INTERNAL);  // inconsistent counts: never write out of bounds
+    }
+    __device__ __forceinline__ void staged(const uint16_t *st, int m, int64_t c) const
+    {
+        const int64_t ce = c + m;
         if (kt.n >= 0) {
             for (int e = 0; e < kt.n; ++e) {
                 const int64_t a0 = c > kt.start[e] ? c : kt.start[e];
                 const int64_t a1 = ce < kt.keep_end[e] ? ce : kt.keep_end[e];
-                if (a0 < a1) {
-                    if (a0 + kt.shift[e] >= 0 && a1 + kt.shift[e] <= N)
-                        store_staged(anc + (a0 + kt.shift[e]), stage + (a0 - c), (int)(a1 - a0), base, n, flags);
-                    else if (threadIdx.x == 0)
-                        atomicOr(const_cast<int32_t *>(flags), FLAG_INTERNAL);  // inconsistent counts: never write out of bounds
-                }
+                if (a0 < a1)
+                    piece(anc, a0 + kt.shift[e], st + (a0 - c), (int)(a1 - a0));
                 const int64_t b0 = c > kt.keep_end[e] ? c : kt.keep_end[e];
                 const int64_t b1 = ce < kt.start[e + 1] ? ce : kt.start[e + 1];
-                if (b0 < b1) {
-                    if (b0 + sent_shift >= 0 && b1 + sent_shift <= N)
-                        store_staged(anc_sys + (b0 + sent_shift), stage + (b0 - c), (int)(b1 - b0), base, n,
-                                     flags);
-                    else if (threadIdx.x == 0)
-                        atomicOr(const_cast<int32_t *>(flags), FLAG_INTERNAL);
-                }
+                if (b0 < b1)
+                    piece(anc_sys, b0 + sent_shift, st + (b0 - c), (int)(b1 - b0));
             }
-        } else {
-            for (int k = threadIdx.x; k < m; k += blockDim.x) {
-                const int64_t j = c + k;
-                int32_t a = 0, b = G - 1;  // the last g with Tg[g] <= j (Tg[0] = 0 <= j)
-                while (a < b) {
-                    const int32_t mid = (a + b + 1) >> 1;
-                    if (__ldg(Tg + mid) <= j)
-                        a = mid;
-                    else
-                        b = mid - 1;
-                }
-                const int64_t s0 = __ldg(Tg + a), o = __ldg(Tg + a + 1) - s0;
-                const int64_t nk = target_of(bl, a);
-                const int64_t keep = o < nk ? o : nk;
-                const int64_t slot = (j - s0 < keep) ? balanced_offset(bl, a) + (j - s0) : j + sent_shift;
-                int32_t *dst = (j - s0 < keep) ? anc : anc_sys;
-                if (slot >= 0 && slot < N && PPF_DCHECK(stage[k] < n, flags, FLAG_INTERNAL))
-                    dst[slot] = base + stage[k];
-                else if (slot < 0 || slot >= N)
-                    atomicOr(const_cast<int32_t *>(flags), FLAG_INTERNAL);
-            }
+            return;
         }
-        __syncthreads();
+        for (int k = threadIdx.x; k < m; k += TILE_THREADS) {
+            const int64_t j = c + k;
+            int32_t a = 0, b = G - 1;  // the last g with Tg[g] <= j (Tg[0] = 0 <= j)
+            while (a < b) {
+                const int32_t mid = (a + b + 1) >> 1;
+                if (__ldg(Tg + mid) <= j)
+                    a = mid;
+                else
+                    b = mid - 1;
+            }
+            const int64_t s0 = __ldg(Tg + a), o = __ldg(Tg + a + 1) - s0;
+            const int64_t nk = target_of(bl, a);
+            const int64_t keep = o < nk ? o : nk;
+            const int64_t slot = (j - s0 < keep) ? balanced_offset(bl, a) + (j - s0) : j + sent_shift;
+            int32_t *dst = (j - s0 < keep) ? anc : anc_sys;
+            if (slot >= 0 && slot < N && PPF_DCHECK(st[k] < n, flags, FLAG_INTERNAL))
+                dst[slot] = base + st[k];
+            else if (slot < 0 || slot >= N)
+                atomicOr(const_cast<int32_t *>(flags), FLAG_INTERNAL);
+        }
     }
-}
+};
 
 // ---------------------------------------------------------------- R3 fill
-// A fill block covers tickets [i_lo, i_hi) of one tile (at most
-// ITEM_TICKETS); the tile's cumulative weights are built once in shared
-// memory, the parents of the tickets are staged there and written out
-// coalesced: to out[j] (systematic, LGS), or split into kept and sent
-// tickets (GS, SGS: kr.anc set).  Dynamic shared memory: FILL_SMEM_BYTES.
+// Block t < T takes tile t's first ITEM_TICKETS tickets, block T + e the e-th
+// entry (t, k) of the list of further runs; a tile without tickets ends its
+// block at once.  The tile's weights are quantised and summed in registers and
+// the parents of the run's tickets drawn among them, straight to out[j]
+// (systematic, LGS) or split into kept and sent tickets (GS, SGS: kr.anc set).
+// Bound by instruction issue (65 thread instructions per particle and ticket,
+// IPC 2.4, 64 registers): 98 us at 38M particles (208 before, with the merge),
+// 22 us at 8M (47); with the kept / sent split 29 us at 8M (52).
 struct KeptRoute {
     int32_t *anc;           // final ancestors; nullptr: every ticket to out[j]
     const int64_t *Tg;      // [G+1] tickets below each group start
@@ -604,28 +588,60 @@ struct KeptRoute {
     Balanced bl;            // the balanced layout GS and SGS leave
 };
 
-// The parents of tickets [i_lo, i_hi) of tile t: the tile's cumulative
-// weights are built once in shared memory, the parents of the tickets are
-// staged there and written out coalesced: to out[j] (systematic, LGS), or
-// split into kept and sent tickets (GS, SGS: kr.anc set).
+struct FillArgs {
+    const float *__restrict__ lw;
+    int64_t N;
+    int32_t T;
+    Divisor ndiv;
+    const DevSummary *__restrict__ sum;
+    const uint64_t *__restrict__ Ct;
+    const int64_t *__restrict__ Tt;
+    const int32_t *__restrict__ To;
+    const uint64_t *__restrict__ St;
+    const int2 *__restrict__ extra;
+    int32_t *__restrict__ out;
+    KeptRoute kr;
+};
+
 template <bool ROUTE>
-__device__ __forceinline__ void fill_tile_tickets(const float *__restrict__ lw, int64_t N, Divisor ndiv,
-                                                  const DevSummary *__restrict__ sum, uint64_t ct, int32_t t,
-                                                  int64_t i_lo, int64_t i_hi, int32_t *__restrict__ out,
-                                                  const KeptRoute &kr)
+__global__ void __launch_bounds__(TILE_THREADS, 4) fill_tiles_kernel(FillArgs A)
 {
-    extern __shared__ uint64_t fill_smem[];
-    uint64_t *C = fill_smem;
-    uint16_t *stage = reinterpret_cast<uint16_t *>(fill_smem + TILE_SMEM_U64);
-    __shared__ uint64_t red[33];
+    const DevSummary *__restrict__ sum = A.sum;
+    // the tile's bounds are read together with the flags that may end the block
+    const int32_t deg = sum->degenerate, n_extra = sum->n_extra;
+    int32_t t = blockIdx.x, k = 0;
+    if (t >= A.T) {
+        if (deg || t - A.T >= n_extra)
+            return;
+        const int2 e = A.extra[t - A.T];
+        t = e.x;
+        k = e.y;
+    }
+    const int64_t tt0 = A.Tt[t], tt1 = A.Tt[t + 1];
+    TicketRun run;
+    run.c0 = A.Ct[t];
+    run.off = A.To[t];
+    run.j_lo = tt0 + (int64_t)k * ITEM_TICKETS;
+    run.L = (int32_t)(tt1 - run.j_lo < ITEM_TICKETS ? tt1 - run.j_lo : ITEM_TICKETS);
+    if (deg || run.L <= 0)
+        return;  // kept by the N_eff test, no usable weight, or a tile without tickets
+    __shared__ ParentSmem sm;
     __shared__ KeptTable kt;
-    const uint64_t sQ = sum->Q, su = sum->u, sqN = sum->qN;
-    const uint32_t sqR = sum->qR;
-    if (ROUTE && threadIdx.x >= blockDim.x - 32) {
-        // the last warp: the groups holding the tile's particles, one lane
-        // each (ga, the group of the tile's first particle, to gb, the last
-        // group starting inside it)
-        const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t N = A.N, lo = (int64_t)t * TILE;
+    const int n = (int)(N - lo < TILE ? N - lo : TILE);
+    float v[TILE_ITEMS];
+    tile_load16(A.lw, N, lo, n, v);
+    const uint64_t below = A.St[(int64_t)t * STRIPS + warp];
+    const TicketScale sc{sum->tsv, sum->tsr, sum->tsl};
+    auto grid = [&]() {  // (read where it is needed, not held in registers)
+        return ticket_grid(__ldcg(&sum->Q), __ldcg(&sum->u), __ldcg(&sum->qN), __ldcg(&sum->qR), A.ndiv);
+    };
+    if (ROUTE && warp == STRIPS - 1) {
+        // the groups holding the tile's particles, one lane each (ga, the
+        // group of the tile's first particle, to gb, the last group starting
+        // inside it)
+        const KeptRoute &kr = A.kr;
         const int32_t gf = __ldg(kr.tile_g + 2 * t), ns = __ldg(kr.tile_g + 2 * t + 1);
         if (ns > GT_MASKED) {
             if (lane == 0)
@@ -635,97 +651,51 @@ __device__ __forceinline__ void fill_tile_tickets(const float *__restrict__ lw, 
             const int ng = gb - ga + 1;
             if (lane <= ng) {
                 const int32_t g = ga + lane;
-                const int64_t s0 = __ldg(kr.Tg + g);
-                kt.start[lane] = s0;
+                const int64_t t0 = __ldg(kr.Tg + g);
+                kt.start[lane] = t0;
                 if (lane < ng) {
-                    const int64_t o = __ldg(kr.Tg + g + 1) - s0, nk = target_of(kr.bl, g);
-                    kt.keep_end[lane] = s0 + (o < nk ? o : nk);
-                    kt.shift[lane] = balanced_offset(kr.bl, g) - s0;
+                    const int64_t o = __ldg(kr.Tg + g + 1) - t0, nk = target_of(kr.bl, g);
+                    kt.keep_end[lane] = t0 + (o < nk ? o : nk);
+                    kt.shift[lane] = balanced_offset(kr.bl, g) - t0;
                 }
             }
             if (lane == 0)
                 kt.n = ng;
         }
     }
-    const int64_t lo = (int64_t)t * TILE;
-    const int n = (int)(N - lo < TILE ? N - lo : TILE);
-    uint64_t q[TILE_ITEMS];
-    tile_weights(lw, lo, n, sum->M, scale_bits(N), C, q);  // its barriers also publish the table
-    tile_scan(q, C, red);
-    const TicketGrid tg = ticket_grid(sQ, su, sqN, sqR, ndiv);
-    if (ROUTE)
-        ticket_parents_routed(C, n, ct, tg, i_lo, i_hi, stage, kt, kr.anc, out, 0, (int32_t)lo, N, kr.G, kr.bl,
-                              kr.Tg, &sum->flags);
+    auto draw = [&](const auto &em) {
+        clear_places(sm, em.lead(run.j_lo), run.L);
+        TileSums ts;
+        tile_quantise(v, sum->M, scale_bits(N), ts);
+        strip_scan(ts, below);
+        if (tt1 - tt0 > ITEM_TICKETS)
+            run = part_run(ts, run.c0, grid(), sc, run.j_lo, run.L);
+        __syncthreads();  // the cleared places and the table
+        block_parents(ts, run, grid, sc, sm, em);
+    };
+    if constexpr (ROUTE)
+        draw(EmitRouted{kt, A.kr.anc, A.out, 0, (int32_t)lo, n, N, A.kr.G, A.kr.bl, A.kr.Tg, &sum->flags});
     else
-        ticket_parents_contig(C, n, ct, tg, i_lo, i_hi, stage, out, (int32_t)lo, N, &sum->flags);
+        draw(EmitContig{A.out, (int32_t)lo, n, N, &sum->flags});
 }
 
-// The fill of the one-block tile scan (the allocation-free entry point): work
-// item b covers tickets [i_lo, i_hi) of one tile (at most ITEM_TICKETS), the
-// tile found from the item map, or by bisection over item_off without it.
-// Dynamic shared memory: FILL_SMEM_BYTES.
-__global__ void __launch_bounds__(TILE_THREADS) fill_kernel(
-    const float *__restrict__ lw, int64_t N, int32_t T, Divisor ndiv, const DevSummary *__restrict__ sum,
-    const uint64_t *__restrict__ Ct, const int64_t *__restrict__ Tt, const int32_t *__restrict__ item_off,
-    const int32_t *__restrict__ item_tile, int32_t *__restrict__ out)
+static cudaError_t launch_fill(const FillArgs &A, cudaStream_t stream)
 {
-    __shared__ int32_t st;
-    const int32_t b = blockIdx.x;
-    // item_tile has an entry for every block of the launch: read it together
-    // with the item count
-    const int32_t t_pre = item_tile ? item_tile[b] : 0;
-    if (b >= sum->n_items)
-        return;
-    if (item_tile == nullptr && threadIdx.x == 0) {
-        int32_t a = 0, e = T;  // last t with item_off[t] <= b
-        while (a < e) {
-            const int32_t mid = (a + e + 1) >> 1;
-            if (item_off[mid] <= b)
-                a = mid;
-            else
-                e = mid - 1;
-        }
-        st = a;
-    }
-    if (item_tile == nullptr)
-        __syncthreads();
-    const int32_t t = item_tile ? t_pre : st;
-    const int64_t tt0 = Tt[t], tt1 = Tt[t + 1];
-    const int64_t i_lo = tt0 + (int64_t)(b - item_off[t]) * ITEM_TICKETS;
-    const int64_t i_hi = (tt1 < i_lo + ITEM_TICKETS) ? tt1 : i_lo + ITEM_TICKETS;
+    const int runs = A.T + (int)(A.N / ITEM_TICKETS) + 1;
+    if (A.kr.anc)
+        fill_tiles_kernel<true><<<runs, TILE_THREADS, 0, stream>>>(A);
+    else
+        fill_tiles_kernel<false><<<runs, TILE_THREADS, 0, stream>>>(A);
+    return cudaGetLastError();
+}
+
+// The fill alone (the allocation-free entry point).
+cudaError_t launch_fill_plain(const float *lw, int64_t N, int32_t T, const DevSummary *sum, const uint64_t *Ct,
+                              const int64_t *Tt, const int32_t *To, const uint64_t *St, const int2 *extra,
+                              int32_t *out, cudaStream_t stream)
+{
     const KeptRoute none{nullptr, nullptr, nullptr, 0, Balanced{0, 0}};
-    fill_tile_tickets<false>(lw, N, ndiv, sum, Ct[t], t, i_lo, i_hi, out, none);
-}
-
-// The fill after tile_tickets_kernel: block t < T takes tile t's first
-// ITEM_TICKETS tickets, block T + e the e-th entry (t, k) of the list of
-// further runs.  A tile without tickets returns at once.
-template <bool ROUTE>
-__global__ void __launch_bounds__(TILE_THREADS) fill_tiles_kernel(
-    const float *__restrict__ lw, int64_t N, int32_t T, Divisor ndiv, const DevSummary *__restrict__ sum,
-    const uint64_t *__restrict__ Ct, const int64_t *__restrict__ Tt, const int2 *__restrict__ extra,
-    int32_t *__restrict__ out, KeptRoute kr)
-{
-    const int32_t b = blockIdx.x;
-    if (sum->degenerate)
-        return;  // kept by the N_eff test, or no usable weight
-    int32_t t, k;
-    if (b < T) {
-        t = b;
-        k = 0;
-    } else {
-        if (b - T >= sum->n_extra)
-            return;
-        const int2 e = extra[b - T];
-        t = e.x;
-        k = e.y;
-    }
-    const int64_t tt0 = Tt[t], tt1 = Tt[t + 1];
-    const int64_t i_lo = tt0 + (int64_t)k * ITEM_TICKETS;
-    const int64_t i_hi = (tt1 < i_lo + ITEM_TICKETS) ? tt1 : i_lo + ITEM_TICKETS;
-    if (i_lo >= i_hi)
-        return;  // a tile without tickets
-    fill_tile_tickets<ROUTE>(lw, N, ndiv, sum, Ct[t], t, i_lo, i_hi, out, kr);
+    return launch_fill(FillArgs{lw, N, T, make_divisor((uint32_t)N), sum, Ct, Tt, To, St, extra, out, none}, stream);
 }
 
 // ------------------------------------------------ two-stage RPA, stage 2
@@ -772,7 +742,8 @@ __global__ void __launch_bounds__(256) group_grid_kernel(
     gg.Q = ce - ca;
     gg.nt = (nt > 0 && gg.Q > 0) ? (uint32_t)nt : 0u;
     gg.u = gg.qN = gg.dm = 0;
-    gg.qR = 0;
+    gg.qR = gg.tsv = 0;
+    gg.tsr = gg.tsl = gg.off = 0;
     gg.p0 = a;
     gg.p1 = e;
     gg.tg0 = Tg[g];
@@ -786,6 +757,11 @@ __global__ void __launch_bounds__(256) group_grid_kernel(
         gg.dm = make_divisor(gg.nt).m;
         gg.qN = gg.Q / gg.nt;
         gg.qR = (uint32_t)(gg.Q % gg.nt);
+        const TicketScale sc = ticket_scale(gg.Q, gg.nt);
+        gg.tsv = sc.v;
+        gg.tsr = sc.sr;
+        gg.tsl = sc.sl;
+        gg.off = run_offset(0, ticket_grid(gg.Q, gg.u, gg.qN, gg.qR, Divisor{gg.dm, gg.nt}), sc, 0, true);
     }
     grid[g] = gg;
     if (gg.nt == 0)
@@ -854,7 +830,7 @@ __device__ __forceinline__ void group_fill_item(const float *__restrict__ lw, in
                                                 int64_t p1, int64_t j0, int64_t j1, int32_t run, uint64_t carry,
                                                 float M, int s, const DevSummary *__restrict__ sum,
                                                 int32_t *__restrict__ out, int32_t *__restrict__ kept_anc,
-                                                const Balanced &bl, uint64_t *C, uint16_t *stage, uint64_t *red)
+                                                const Balanced &bl, ParentSmem &sm)
 {
     const int64_t nt = gg.nt;
     Divisor dv;
@@ -865,16 +841,16 @@ __device__ __forceinline__ void group_fill_item(const float *__restrict__ lw, in
     kt.n = 1;
     kt.start[0] = 0;
     kt.start[1] = nt;
-    kt.keep_end[0] = gg.keep;
+    kt.keep_end[0] = kept_anc ? gg.keep : 0;  // LGS: every ticket to its ticket slot
     kt.shift[0] = gg.shift;
     // chunks of at most TILE particles; the local tickets of a chunk with
     // cumulative weight [carry, carry + total) inside the group are
     // [T(carry), T(carry + total)), T the count below of the nt tickets
     for (int64_t c0 = p0; c0 < p1; c0 += TILE) {
         const int n = (int)(p1 - c0 < TILE ? p1 - c0 : TILE);
-        uint64_t q[TILE_ITEMS];
-        tile_weights(lw, c0, n, M, s, C, q);
-        const uint64_t tot = tile_scan(q, C, red);
+        TileSums ts;
+        tile_sums(lw, N, c0, n, M, s, ts, sm);
+        const uint64_t tot = tile_total(sm);
         // no ticket lies below the group's start, all of them below its end
         const int64_t c_lo = carry == 0 ? 0 : tickets_below(carry, nt, gg.u, gg.Q);
         const int64_t c_hi = c0 + n == gg.p1 ? nt : tickets_below(carry + tot, nt, gg.u, gg.Q);
@@ -886,12 +862,19 @@ __device__ __forceinline__ void group_fill_item(const float *__restrict__ lw, in
             t_lo = c_lo > j0 ? c_lo : j0;
             t_hi = c_hi < j1 ? c_hi : j1;
         }
-        if (kept_anc)
-            ticket_parents_routed(C, n, carry, tg, t_lo, t_hi, stage, kt, kept_anc, out, gg.tg0, (int32_t)c0, N, G,
-                                  bl, Tg, &sum->flags);
-        else
-            ticket_parents_contig(C, n, carry, tg, t_lo, t_hi, stage, out + gg.tg0, (int32_t)c0,
-                                  (nt < N - gg.tg0) ? nt : N - gg.tg0, &sum->flags);
+        if (t_lo < t_hi) {  // (at most ITEM_TICKETS: one run)
+            const TicketScale sc{gg.tsv, gg.tsr, gg.tsl};
+            const int L = (int)(t_hi - t_lo);
+            clear_places(sm, 0, L);
+            TicketRun rn{carry, t_lo, L, gg.off};
+            if (t_lo != c_lo || t_hi != c_hi)
+                rn = part_run(ts, carry, tg, sc, t_lo, L);
+            else if (carry > 0)
+                rn.off = run_offset(carry, tg, sc, t_lo, true);
+            __syncthreads();
+            block_parents(ts, rn, [&]() { return tg; }, sc, sm,
+                          EmitRouted{kt, kept_anc, out, gg.tg0, (int32_t)c0, n, N, G, bl, Tg, &sum->flags});
+        }
         carry += tot;
         __syncthreads();
     }
@@ -901,16 +884,13 @@ __device__ __forceinline__ void group_fill_item(const float *__restrict__ lw, in
 // n_workers + g takes a small group g whole, or its first ITEM_TICKETS
 // tickets when it is heavy (a large group is all in the split list).
 // s: scale_bits(N).
-__global__ void __launch_bounds__(TILE_THREADS, 4) group_fill_kernel(
+__global__ void __launch_bounds__(TILE_THREADS, 3) group_fill_kernel(
     const float *__restrict__ lw, int64_t N, int32_t G, const int64_t *__restrict__ Tg,
     const uint64_t *__restrict__ Ct, const GroupGrid *__restrict__ grid, const int4 *__restrict__ split,
     int32_t n_workers, const DevSummary *__restrict__ sum, double ess_thr, int32_t *__restrict__ out,
     int32_t *__restrict__ kept_anc, Balanced bl, int s)
 {
-    extern __shared__ uint64_t fill_smem[];  // FILL_SMEM_BYTES
-    uint64_t *C = fill_smem;
-    uint16_t *stage = reinterpret_cast<uint16_t *>(fill_smem + TILE_SMEM_U64);
-    __shared__ uint64_t red[33];
+    __shared__ ParentSmem sm;
     if ((int32_t)blockIdx.x >= n_workers) {  // a group block: one item, no loop
         const GroupGrid gg = grid[blockIdx.x - n_workers];
         const double ess = sum->ess;
@@ -919,8 +899,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 4) group_fill_kernel(
         if (ess >= ess_thr || deg || gg.nt == 0 || gg.p1 - gg.p0 > GROUP_SPLIT)
             return;  // kept by the N_eff test, no usable weight, no offspring, or a large group
         const int64_t j1 = gg.nt > ITEM_TICKETS ? ITEM_TICKETS : gg.nt;  // a heavy group's first run
-        group_fill_item(lw, N, G, Tg, gg, gg.p0, gg.p1, 0, j1, -1, 0, M, s, sum, out, kept_anc, bl, C, stage,
-                        red);
+        group_fill_item(lw, N, G, Tg, gg, gg.p0, gg.p1, 0, j1, -1, 0, M, s, sum, out, kept_anc, bl, sm);
         return;
     }
     if (sum->ess >= ess_thr || sum->degenerate)
@@ -934,13 +913,11 @@ __global__ void __launch_bounds__(TILE_THREADS, 4) group_fill_kernel(
             int64_t p0, p1;
             uint64_t carry;
             tile_part(gg, en.x, Ct, p0, p1, carry);
-            group_fill_item(lw, N, G, Tg, gg, p0, p1, 0, 0, en.z, carry, M, s, sum, out, kept_anc, bl, C, stage,
-                            red);
+            group_fill_item(lw, N, G, Tg, gg, p0, p1, 0, 0, en.z, carry, M, s, sum, out, kept_anc, bl, sm);
         } else {  // run en.z of a heavy small group
             const int64_t j0 = (int64_t)en.z * ITEM_TICKETS;
             const int64_t j1 = (j0 + ITEM_TICKETS < (int64_t)gg.nt) ? j0 + ITEM_TICKETS : (int64_t)gg.nt;
-            group_fill_item(lw, N, G, Tg, gg, gg.p0, gg.p1, j0, j1, -1, 0, M, s, sum, out, kept_anc, bl, C, stage,
-                            red);
+            group_fill_item(lw, N, G, Tg, gg, gg.p0, gg.p1, j0, j1, -1, 0, M, s, sum, out, kept_anc, bl, sm);
         }
     }
 }
@@ -1599,28 +1576,101 @@ __global__ void __launch_bounds__(256) route_copy_kernel(const int32_t *__restri
 }
 
 // ------------------------------------------------------------------- RNA
+// A group's offspring: ticket s2 goes to the group's own slot lo + s2, the last
+// mig of them to the tail of the next group of the ring (at `tail`).
+struct EmitRing {
+    static constexpr bool DIRECT = false;
+    int32_t *__restrict__ anc;
+    float *__restrict__ lwp;
+    float lwg;
+    int32_t base;
+    int n;
+    int64_t lo, keep, tail, N;  // own slots [lo, lo + keep), then tail ..
+    const int32_t *flags;
+    __device__ __forceinline__ int lead(int64_t) const { return 0; }
+    // m offspring to the slots from d on, their weight beside them
+    __device__ __forceinline__ void piece(int64_t d, const uint16_t *st, int m) const
+    {
+        if (!PPF_DCHECK(d >= 0 && d + m <= N, flags, FLAG_INTERNAL))
+            return;
+        store_staged(anc + d, st, m, base, n, flags);
+        float *o = lwp + d;
+        const int head = (int)((4u - ((uint32_t)(reinterpret_cast<uintptr_t>(o) >> 2) & 3u)) & 3u);
+        const int h = head < m ? head : m, m4 = (m - h) >> 2, t0 = h + 4 * m4, k = threadIdx.x;
+        if (k < h)
+            o[k] = lwg;
+        for (int q = k; q < m4; q += blockDim.x)
+            reinterpret_cast<float4 *>(o + h)[q] = make_float4(lwg, lwg, lwg, lwg);
+        if (k < m - t0)
+            o[t0 + k] = lwg;
+    }
+    __device__ __forceinline__ void staged(const uint16_t *st, int m, int64_t c) const
+    {
+        const int own = c < keep ? (keep - c < m ? (int)(keep - c) : m) : 0;
+        if (own > 0)
+            piece(lo + c, st, own);
+        if (own < m)
+            piece(tail + (c + own - keep), st + own, m - own);
+    }
+};
+
+// The draw of a group larger than the block's 16 NT particles, in chunks of
+// them; the tickets of a chunk are [T(carry), T(carry + total)), T the count
+// below of the group's sz tickets.  (A call: its registers stay out of the
+// kernel's common path.)
+template <int NT>
+static __device__ __noinline__ void rna_chunks(const float *__restrict__ lw, int64_t N, int64_t lo, int64_t sz, float Mg,
+                                               int s, TicketGrid tg, TicketScale sc, ParentSmemT<NT> *sm, EmitRing em)
+{
+    constexpr int PART = NT * TILE_ITEMS;
+    uint64_t carry = 0;
+    for (int64_t c0 = 0; c0 < sz; c0 += PART) {
+        const int n = (int)(sz - c0 < PART ? sz - c0 : PART);
+        TileSums ts;
+        tile_sums(lw, N, lo + c0, n, Mg, s, ts, *sm);
+        const uint64_t tot = tile_total(*sm);
+        const int64_t t_lo = tickets_below(carry, sz, tg.u, tg.Q);
+        const int64_t t_hi = tickets_below(carry + tot, sz, tg.u, tg.Q);
+        em.base = (int32_t)(lo + c0);
+        em.n = n;
+        draw_parents(ts, carry, tg, sc, t_lo, t_hi, true, run_offset(carry, tg, sc, t_lo, true), *sm, em,
+                     [&](TileSums &t) { tile_sums(lw, N, lo + c0, n, Mg, s, t, *sm); });
+        carry += tot;
+        __syncthreads();
+    }
+}
+
 // One block per group: group max, fixed-point weights, local total and group
 // weight (FP64 against the global total of the step), local systematic
 // tickets, then every offspring is written to its slot -- the last `mig`
 // slots of the group go to the tail of the next group of the ring (group
 // g + 1 mod G, or succ[g] for ARNA's ring).
-__global__ void __launch_bounds__(TILE_THREADS, 4) rna_kernel(
+//
+// NT threads hold 16 NT particles: 64 for groups up to 1024, 128 up to 2048,
+// else 256 (so that a small group does not leave most warps idle at the
+// barriers).  Sums of e^(lw - Mg) are taken in one order for every NT: as if
+// by 256 threads in strides of 256, lane sums by the warps' butterfly, the 8
+// warps in turn.  Bound by the block's chain of barriers and its FP64
+// logarithms (two per group: two lanes take one each): 20.6 us at 3.1M
+// particles in groups of 4001 (31.5 before), 16.2 us at 2M (20.6).
+template <int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT - 1) rna_kernel(
     const float *__restrict__ lw, int64_t N, int32_t G, const int64_t *__restrict__ goff,
     const int32_t *__restrict__ succ, DevSummary *sum, double ess_thr, uint64_t seed, uint32_t fid, uint32_t frame,
-    int32_t *__restrict__ anc, float *__restrict__ lwp)
+    int32_t *__restrict__ anc, float *__restrict__ lwp, Divisor d_small, Divisor d_large)
 {
     if (kept_by_ess(sum, ess_thr))
         return;
     const int64_t mig = sum->mig;
-    extern __shared__ uint64_t fill_smem[];  // FILL_SMEM_BYTES
-    uint64_t *C = fill_smem;
-    uint16_t *stage = reinterpret_cast<uint16_t *>(fill_smem + TILE_SMEM_U64);
-    __shared__ uint64_t red[33];
+    constexpr int NW = NT / 32, VT = 256 / NT;  // virtual threads of the 256 per thread
+    __shared__ ParentSmemT<NT> sm;
     __shared__ float smf[8];
-    __shared__ double lwg_s;
+    __shared__ float lwg_s;
     __shared__ uint64_t Qs, us, qNs;
     __shared__ uint32_t qRs;
     __shared__ Divisor dvs;
+    __shared__ TicketScale scs;
+    __shared__ int32_t offs;
     const int32_t g = blockIdx.x;
     const int64_t lo = goff[g], sz = goff[g + 1] - lo;
     if (sz <= 0)
@@ -1628,161 +1678,130 @@ __global__ void __launch_bounds__(TILE_THREADS, 4) rna_kernel(
     const int32_t gn = succ ? succ[g] : (g + 1) % G;
     const int64_t gn_lo = goff[gn], gn_sz = goff[gn + 1] - gn_lo;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    auto dest = [&](int64_t s2) -> int64_t {
-        return (s2 < sz - mig) ? lo + s2 : gn_lo + gn_sz - mig + (s2 - (sz - mig));
-    };
-    if (sz <= TILE) {
-        // the whole group in one tile: its weights are loaded once and kept
-        // in registers for the maximum, the sum of e^(lw - Mg), and the
-        // quantised scan (whose total is the group's Q)
-        const int n = (int)sz;
-        float v[TILE_LOADS];
-        tile_load(lw, lo, n, v);
-        float m = -INFINITY;
-#pragma unroll
-        for (int k = 0; k < TILE_LOADS; ++k)
-            m = fmaxf(m, v[k]);
+    const EmitRing em{anc, lwp, 0.0f, (int32_t)lo, (int)(sz < TILE ? sz : TILE), lo, sz - mig, gn_lo + gn_sz - mig, N,
+                      &sum->flags};
+    const bool one = sz <= NT * TILE_ITEMS;  // the whole group in the block's registers
+    const int s = scale_bits(sz);
+    float Mg = -INFINITY;
+    auto group_max = [&](float m) {
         m = warp_max(m);
         if (lane == 0)
             smf[warp] = m;
         __syncthreads();
-        float Mg = -INFINITY;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
+        for (int w = 0; w < NW; ++w)
             Mg = fmaxf(Mg, smf[w]);
-        float es = 0.0f;
-#pragma unroll
-        for (int k = 0; k < TILE_LOADS; ++k)
-            if (v[k] > -INFINITY)
-                es += __expf(v[k] - Mg);
-        es = warp_sum(es);
         __syncthreads();  // every thread has read smf
+    };
+    TileSums ts;
+    uint64_t q_all = 0;
+    if (one) {
+        // loaded in strides for the maximum and the sum of e^(lw - Mg), then
+        // consecutively, from L1, for the quantised scan (whose total is the
+        // group's Q)
+        const int n = (int)sz;
+        constexpr int PER = TILE_ITEMS / VT;
+        float v[TILE_ITEMS];
+        float m = -INFINITY;
+#pragma unroll
+        for (int j = 0; j < VT; ++j)
+#pragma unroll
+            for (int k = 0; k < PER; ++k) {
+                const int e = (int)threadIdx.x + j * NT + k * 256;
+                v[j * PER + k] = (e < n) ? __ldg(lw + lo + e) : -INFINITY;
+                m = fmaxf(m, v[j * PER + k]);
+            }
+        group_max(m);
+#pragma unroll
+        for (int j = 0; j < VT; ++j) {
+            float es = 0.0f;
+#pragma unroll
+            for (int k = 0; k < PER; ++k)
+                if (v[j * PER + k] > -INFINITY)
+                    es += __expf(v[j * PER + k] - Mg);
+            es = warp_sum(es);
+            if (lane == 0)
+                smf[warp + j * NW] = es;
+        }
+        tile_load16(lw, N, lo, n, v);
+        tile_quantise(v, Mg, s, ts);
+        clear_places(sm, 0, n);
+        tile_scan(ts, sm);  // its barrier also publishes smf and the cleared places
+        q_all = tile_total(sm);
+    } else {
+        float m = -INFINITY;
+        for (int64_t i = threadIdx.x; i < sz; i += NT)
+            m = fmaxf(m, __ldg(lw + lo + i));
+        group_max(m);
+        uint64_t qs = 0;
+        for (int j = 0; j < VT; ++j) {
+            float es = 0.0f;
+            for (int64_t i = threadIdx.x + j * NT; i < sz; i += 512) {
+                // two strided elements at a time
+                const int64_t i2 = i + 256;
+                const float v = __ldg(lw + lo + i);
+                const float w = (i2 < sz) ? __ldg(lw + lo + i2) : -INFINITY;
+                uint64_t a, b;
+                quantise2(v, w, Mg, s, a, b);
+                qs += a + b;
+                if (v > -INFINITY)
+                    es += __expf(v - Mg);
+                if (w > -INFINITY)
+                    es += __expf(w - Mg);
+            }
+            es = warp_sum(es);
+            if (lane == 0)
+                smf[warp + j * NW] = es;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            qs += __shfl_xor_sync(0xffffffffu, qs, o);
         if (lane == 0)
-            smf[warp] = es;
-        const int s = scale_bits(sz);
-        uint64_t q[TILE_ITEMS];
-        tile_quantise(v, Mg, s, C, q);  // its barriers also publish smf
-        const uint64_t Qg = tile_scan(q, C, red);
-        if (threadIdx.x == 0) {
-            float e = 0.0f;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
-                e += smf[w];
-            dvs = make_divisor((uint32_t)sz);
-            qNs = Qg / (uint64_t)sz;
-            qRs = (uint32_t)(Qg % (uint64_t)sz);
-            if (Qg == 0ull) {
-                lwg_s = -INFINITY;
-                us = 0ull;
-            } else {
-                lwg_s = ((double)Mg + log((double)e)) - sum->log_total - log((double)sz);
-                us = ticket_offset(seed, fid, frame, PURPOSE_GROUP, (uint32_t)g, Qg);
-            }
-        }
+            sm.red[warp] = qs;
         __syncthreads();
-        const float lwg = (float)lwg_s;
-        if (Qg == 0ull) {  // no usable weight in the group: it keeps its slots
-            for (int64_t s2 = threadIdx.x; s2 < sz; s2 += blockDim.x) {
-                const int64_t d = dest(s2);
-                if (!PPF_DCHECK(d >= 0 && d < N, &sum->flags, FLAG_INTERNAL))
-                    continue;
-                anc[d] = (int32_t)(lo + s2);
-                lwp[d] = lwg;
-            }
-            return;
-        }
-        const TicketGrid tg = ticket_grid(Qg, us, qNs, qRs, dvs);
-        ticket_parents_staged(C, n, 0, tg, 0, sz, stage, [&](int64_t j, int i) {
-            const int64_t d = dest(j);
-            if (!PPF_DCHECK(d >= 0 && d < N && i >= 0 && i < n, &sum->flags, FLAG_INTERNAL))
-                return;
-            anc[d] = (int32_t)(lo + i);
-            lwp[d] = lwg;
-        });
-        return;
+        q_all = tile_total(sm);
     }
-    // pass 1: group maximum
-    float m = -INFINITY;
-    for (int64_t i = threadIdx.x; i < sz; i += blockDim.x)
-        m = fmaxf(m, __ldg(lw + lo + i));
-    m = warp_max(m);
-    if (lane == 0)
-        smf[warp] = m;
-    __syncthreads();
-    float Mg = -INFINITY;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
-        Mg = fmaxf(Mg, smf[w]);
-    __syncthreads();
-    const int s = scale_bits(sz);
-    // pass 2: total fixed-point weight and sum of e^(lw - Mg)
-    uint64_t qs = 0;
-    float es = 0.0f;
-    for (int64_t i = threadIdx.x; i < sz; i += 2 * (int64_t)blockDim.x) {
-        // two strided elements at a time (the sum of e^(lw - Mg) keeps its order)
-        const int64_t i2 = i + blockDim.x;
-        const float v = __ldg(lw + lo + i);
-        const float w = (i2 < sz) ? __ldg(lw + lo + i2) : -INFINITY;
-        uint64_t a, b;
-        quantise2(v, w, Mg, s, a, b);
-        qs += a + b;
-        if (v > -INFINITY)
-            es += __expf(v - Mg);
-        if (w > -INFINITY)
-            es += __expf(w - Mg);
-    }
-    uint64_t Qg;
-    block_excl_scan_u64(qs, red, &Qg);
-    es = warp_sum(es);
-    if (lane == 0)
-        smf[warp] = es;
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    // the group's draw: the FP64 weight by two lanes of warp 0 (one logarithm
+    // each), the ticket grid by warp 1
+    if (warp == 0) {
         float e = 0.0f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
+        for (int w = 0; w < 8; ++w)
             e += smf[w];
-        Qs = Qg;
-        dvs = make_divisor((uint32_t)sz);
-        qNs = Qg / (uint64_t)sz;
-        qRs = (uint32_t)(Qg % (uint64_t)sz);
-        if (Qg == 0ull) {
-            lwg_s = -INFINITY;
-            us = 0ull;
-        } else {
-            lwg_s = ((double)Mg + log((double)e)) - sum->log_total - log((double)sz);
-            us = ticket_offset(seed, fid, frame, PURPOSE_GROUP, (uint32_t)g, Qg);
+        const double lg = log(lane == 1 ? (double)sz : (double)e);
+        const double lsz = __shfl_sync(0xffffffffu, lg, 1);
+        if (lane == 0)
+            lwg_s = q_all == 0ull ? -INFINITY : (float)(((double)Mg + lg) - sum->log_total - lsz);
+    }
+    if (threadIdx.x == 32) {
+        Qs = q_all;
+        dvs = sz == (int64_t)d_small.d ? d_small : (sz == (int64_t)d_large.d ? d_large : make_divisor((uint32_t)sz));
+        uint32_t r;
+        qNs = div_by(q_all, dvs, &r);
+        qRs = r;
+        us = 0ull;
+        if (q_all != 0ull) {
+            us = ticket_offset(seed, fid, frame, PURPOSE_GROUP, (uint32_t)g, q_all);
+            scs = ticket_scale(q_all, (uint32_t)sz);
+            offs = run_offset(0, ticket_grid(q_all, us, qNs, qRs, dvs), scs, 0, true);
         }
     }
     __syncthreads();
-    const uint64_t Q = Qs, u = us;
-    const float lwg = (float)lwg_s;
-    if (Q == 0ull) {  // no usable weight in the group: it keeps its slots
-        for (int64_t s2 = threadIdx.x; s2 < sz; s2 += blockDim.x) {
-            const int64_t d = dest(s2);
+    EmitRing ring = em;
+    ring.lwg = lwg_s;
+    if (q_all == 0ull) {  // no usable weight in the group: it keeps its slots
+        for (int64_t s2 = threadIdx.x; s2 < sz; s2 += NT) {
+            const int64_t d = s2 < em.keep ? lo + s2 : em.tail + (s2 - em.keep);
             if (!PPF_DCHECK(d >= 0 && d < N, &sum->flags, FLAG_INTERNAL))
                 continue;
             anc[d] = (int32_t)(lo + s2);
-            lwp[d] = lwg;
+            lwp[d] = ring.lwg;
         }
         return;
     }
-    const TicketGrid tg = ticket_grid(Q, u, qNs, qRs, dvs);
-    // pass 3: chunks of TILE particles; the tickets of chunk [c0, c0 + n) are
-    // [T(carry), T(carry + total)) with T the local ticket count of n = sz.
-    uint64_t carry = 0;
-    for (int64_t c0 = 0; c0 < sz; c0 += TILE) {
-        const int n = (int)(sz - c0 < TILE ? sz - c0 : TILE);
-        uint64_t q[TILE_ITEMS];
-        tile_weights(lw, lo + c0, n, Mg, s, C, q);
-        const uint64_t tot = tile_scan(q, C, red);
-        const int64_t t_lo = tickets_below(carry, sz, u, Q);
-        const int64_t t_hi = tickets_below(carry + tot, sz, u, Q);
-        ticket_parents_staged(C, n, carry, tg, t_lo, t_hi, stage, [&](int64_t j, int i) {
-            const int64_t d = dest(j);
-            if (!PPF_DCHECK(d >= 0 && d < N && i >= 0 && i < n, &sum->flags, FLAG_INTERNAL))
-                return;
-            anc[d] = (int32_t)(lo + c0 + i);
-            lwp[d] = lwg;
-        });
-        carry += tot;
-        __syncthreads();
+    if (one) {
+        const TicketRun run{0, 0, (int32_t)sz, offs};  // one ticket per particle: one run
+        block_parents(ts, run, [&]() { return ticket_grid(Qs, us, qNs, qRs, dvs); }, scs, sm, ring);
+    } else {
+        rna_chunks<NT>(lw, N, lo, sz, Mg, s, ticket_grid(Qs, us, qNs, qRs, dvs), scs, &sm, ring);
     }
 }
 
@@ -1940,19 +1959,7 @@ __global__ void fill_f32_kernel(float *__restrict__ a, int64_t N, float v)
 // device; called when a context is created).
 cudaError_t resample_kernel_attributes()
 {
-    cudaError_t e = cudaFuncSetAttribute(fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)FILL_SMEM_BYTES);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(fill_tiles_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)FILL_SMEM_BYTES);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(fill_tiles_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)FILL_SMEM_BYTES);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(rna_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FILL_SMEM_BYTES);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(group_fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)FILL_SMEM_BYTES);
+    cudaError_t e = cudaSuccess;
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(schedule_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)SORT_SMEM_BYTES);
@@ -1978,13 +1985,13 @@ static void launch_tile_tickets(ppf_ctx *c, double ess_thr, int rpa)
     // (one launch less); beyond, one thread per tile and group does
     const bool one_block = T <= 1024 && (!rpa || c->G <= 1024);
     tile_scan_kernel<<<1, 1024, sizeof(uint64_t) * (st_tiles + 1), c->stream>>>(
-        c->N, T, c->sc.Qt, c->sc.Ct, c->sc.Tt, c->sc.item_off, nullptr, c->sum, ess_thr, c->m.seed, c->m.filter_id,
-        (uint32_t)c->last_frame, c->goff, c->G, rpa, c->sc.Cbl, c->sc.Tg, st_tiles, nd, one_block ? 0 : 1, extra);
+        c->N, T, c->sc.Qt, c->sc.Ct, c->sc.Tt, c->sum, ess_thr, c->m.seed, c->m.filter_id,
+        (uint32_t)c->last_frame, c->goff, c->G, rpa, c->sc.Cbl, c->sc.Tg, st_tiles, nd, one_block ? 0 : 1, extra, c->sc.To);
     if (one_block)
         return;
     const int n = (rpa && c->G > T ? c->G : T) + 1;
     tile_tickets_kernel<<<(n + 255) / 256, 256, 0, c->stream>>>(c->N, T, c->sc.Ct, c->sc.Tt, c->sum, nd, c->goff,
-                                                                c->G, rpa, c->sc.Cbl, c->sc.Tg, extra);
+                                                                c->G, rpa, c->sc.Cbl, c->sc.Tg, extra, c->sc.To);
     c->launches += 1;
 }
 
@@ -2029,11 +2036,11 @@ cudaError_t launch_resample_global(ppf_ctx *c, int scheme, double ess_thr)
     prof_mark(c, PH_RESAMPLE, 0);
     c->launches += rpa ? 5 : 3;
     if (rpa)
-        tile_group_totals_kernel<<<T, TILE_THREADS, 0, c->stream>>>(lw, c->N, c->sum, ess_thr, c->sc.Qt, c->goff,
-                                                                    c->G, c->sc.Cbl, c->sc.tile_g);
+        tile_group_totals_kernel<<<T, TILE_THREADS, 0, c->stream>>>(lw, c->N, c->sum, ess_thr, c->sc.Qt, c->sc.St,
+                                                                    c->goff, c->G, c->sc.Cbl, c->sc.tile_g);
     else  // five blocks per SM (47 registers), each tile's loads one tile ahead
         tile_totals_kernel<<<T < 5 * c->num_sms ? T : 5 * c->num_sms, TILE_THREADS, 0, c->stream>>>(
-            lw, c->N, c->sum, ess_thr, c->sc.Qt);
+            lw, c->N, c->sum, ess_thr, c->sc.Qt, c->sc.St);
     launch_tile_tickets(c, ess_thr, rpa ? 1 : 0);
     int32_t *out = rpa ? c->anc_sys : c->anc;
     const bool two_stage = (scheme >= PPF_RPA2_GS && scheme <= PPF_RPA2_LGS);
@@ -2054,23 +2061,15 @@ cudaError_t launch_resample_global(ppf_ctx *c, int scheme, double ess_thr)
             (uint32_t)c->last_frame, c->sc.ggrid, split, balanced_layout(c->N, c->G));
         split_runs_kernel<<<c->num_sms, 256, 0, c->stream>>>(c->sc.Ct, c->sc.ggrid, split, c->sum, ess_thr);
         const int n_workers = 4 * c->num_sms;
-        group_fill_kernel<<<n_workers + c->G, TILE_THREADS, FILL_SMEM_BYTES, c->stream>>>(
+        group_fill_kernel<<<n_workers + c->G, TILE_THREADS, 0, c->stream>>>(
             lw, c->N, c->G, c->sc.Tg, c->sc.Ct, c->sc.ggrid, split, n_workers, c->sum, ess_thr, out,
             kept_direct ? c->anc : nullptr, balanced_layout(c->N, c->G), scale_bits(c->N));
         c->launches += 2;
     } else {
-        // block t < T: tile t's first run of tickets; the rest: the listed further runs
-        const int max_items = T + (int)(c->N / ITEM_TICKETS) + 1;
-        const int2 *extra = reinterpret_cast<const int2 *>(c->sc.extra);
-        if (kept_direct) {
-            const KeptRoute kr{c->anc, c->sc.Tg, c->sc.tile_g, c->G, balanced_layout(c->N, c->G)};
-            fill_tiles_kernel<true><<<max_items, TILE_THREADS, FILL_SMEM_BYTES, c->stream>>>(
-                lw, c->N, T, make_divisor((uint32_t)c->N), c->sum, c->sc.Ct, c->sc.Tt, extra, out, kr);
-        } else {
-            const KeptRoute none{nullptr, nullptr, nullptr, 0, Balanced{0, 0}};
-            fill_tiles_kernel<false><<<max_items, TILE_THREADS, FILL_SMEM_BYTES, c->stream>>>(
-                lw, c->N, T, make_divisor((uint32_t)c->N), c->sum, c->sc.Ct, c->sc.Tt, extra, out, none);
-        }
+        const KeptRoute kr{kept_direct ? c->anc : nullptr, c->sc.Tg, c->sc.tile_g, c->G, balanced_layout(c->N, c->G)};
+        const FillArgs A{lw, c->N, T, make_divisor((uint32_t)c->N), c->sum, c->sc.Ct, c->sc.Tt, c->sc.To, c->sc.St,
+                         reinterpret_cast<const int2 *>(c->sc.extra), out, kr};
+        launch_fill(A, c->stream);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || !rpa) {
@@ -2089,14 +2088,31 @@ cudaError_t launch_resample_global(ppf_ctx *c, int scheme, double ess_thr)
     return cudaGetLastError();
 }
 
-cudaError_t launch_resample_rna(ppf_ctx *c, float alpha, double ess_thr)
+// RNA's per-group kernel, the block sized by the balanced groups (any layout
+// is drawn right; groups beyond the block's particles go in chunks).
+static void launch_rna(ppf_ctx *c, double ess_thr, const int32_t *succ)
 {
     const float *lw = c->state[c->cur] + 5 * c->N;
+    const Balanced bl = balanced_layout(c->N, c->G);
+    const Divisor d0 = make_divisor((uint32_t)(bl.q > 0 ? bl.q : 1)), d1 = make_divisor((uint32_t)(bl.q + 1));
+    const int64_t top = c->uneven ? TILE : bl.q + (bl.r > 0 ? 1 : 0);
+    auto go = [&](auto kernel, int nt) {
+        kernel<<<c->G, nt, 0, c->stream>>>(lw, c->N, c->G, c->goff, succ, c->sum, ess_thr, c->m.seed, c->m.filter_id,
+                                           (uint32_t)c->last_frame, c->anc, c->lwp, d0, d1);
+    };
+    if (top <= 64 * TILE_ITEMS)
+        go(rna_kernel<64>, 64);
+    else if (top <= 128 * TILE_ITEMS)
+        go(rna_kernel<128>, 128);
+    else
+        go(rna_kernel<256>, 256);
+}
+
+cudaError_t launch_resample_rna(ppf_ctx *c, float alpha, double ess_thr)
+{
     prof_mark(c, PH_RESAMPLE, 0);
     rna_prep_kernel<<<1, 1024, 0, c->stream>>>(c->goff, c->G, alpha, c->sum, ess_thr);
-    rna_kernel<<<c->G, TILE_THREADS, FILL_SMEM_BYTES, c->stream>>>(lw, c->N, c->G, c->goff, nullptr, c->sum, ess_thr,
-                                                                   c->m.seed, c->m.filter_id,
-                                                                   (uint32_t)c->last_frame, c->anc, c->lwp);
+    launch_rna(c, ess_thr, nullptr);
     prof_mark(c, PH_RESAMPLE, 1);
     c->launches += 2;
     return cudaGetLastError();
@@ -2109,15 +2125,13 @@ cudaError_t launch_resample_arna(ppf_ctx *c, float alpha, double ess_thr)
     const float *lw = c->state[c->cur] + 5 * c->N;
     const int T = c->T;
     prof_mark(c, PH_RESAMPLE, 0);
-    tile_group_totals_kernel<<<T, TILE_THREADS, 0, c->stream>>>(lw, c->N, c->sum, ess_thr, c->sc.Qt, c->goff, c->G,
-                                                                c->sc.Cbl, c->sc.tile_g);
+    tile_group_totals_kernel<<<T, TILE_THREADS, 0, c->stream>>>(lw, c->N, c->sum, ess_thr, c->sc.Qt, c->sc.St, c->goff,
+                                                                c->G, c->sc.Cbl, c->sc.tile_g);
     launch_tile_tickets(c, ess_thr, 2);
     arna_prep_kernel<<<1, 1024, sort_smem_bytes(c->G), c->stream>>>(
         c->goff, c->G, alpha, c->sum, ess_thr, c->sc.Tg, c->ring, c->succ, c->m.seed, c->m.filter_id,
         (uint32_t)c->last_frame);
-    rna_kernel<<<c->G, TILE_THREADS, FILL_SMEM_BYTES, c->stream>>>(lw, c->N, c->G, c->goff, c->succ, c->sum, ess_thr,
-                                                                   c->m.seed, c->m.filter_id,
-                                                                   (uint32_t)c->last_frame, c->anc, c->lwp);
+    launch_rna(c, ess_thr, c->succ);
     prof_mark(c, PH_RESAMPLE, 1);
     c->launches += 4;
     return cudaGetLastError();
