@@ -339,19 +339,23 @@ __global__ void batch_finalize_kernel(const Partial *__restrict__ part, const in
         if (q.mp > -INFINITY)
             t[7] += q.sp * (double)expf(q.mp - mp);
     }
-    for (int c = 0; c < 8; ++c)
-        t[c] = warp_sum_d(t[c]);
-    if (lane == 0) {
-        FilterSummary s;
-        for (int c = 0; c < 5; ++c)
-            s.mean[c] = t[1 + c] / t[0];
-        s.ess = t[0] * t[0] / t[6];
-        s.log_evidence = ((double)m + log(t[0])) - ((double)mp + log(t[7]));
-        s.M = m;
-        s.degenerate = (t[0] > 0.0) ? 0 : 1;
-        fs[f] = s;
-        if (cur->est)
-            cur->est[(int64_t)cur->t * F + f] = s;
+    // lane c takes the c-th total
+    double tot = warp_sum8_d(t);
+    tot = __shfl_sync(0xffffffffu, tot, ((lane & 4) << 2) | ((lane & 2) << 2) | ((lane & 1) << 2));
+    const Finish fin = finish_totals(tot, m, mp);
+    FilterSummary *run = cur->est ? cur->est + (int64_t)cur->t * F + f : nullptr;
+    for (FilterSummary *s : {fs + f, run}) {
+        if (!s)
+            continue;
+        if (lane >= 1 && lane <= 5)
+            s->mean[lane - 1] = fin.q;
+        if (lane == 6)
+            s->ess = fin.q;
+        if (lane == 0) {
+            s->log_evidence = fin.log_evidence;
+            s->M = m;
+            s->degenerate = (tot > 0.0) ? 0 : 1;
+        }
     }
 }
 

@@ -17,6 +17,7 @@
 
 #include "ppf_device.cuh"
 #include "ppf_internal.h"
+#include "ppf_kernels.cuh"
 
 namespace ppf {
 
@@ -214,7 +215,7 @@ struct GAcc {
 __device__ void grad_finalize(const GradPartial *part, int n, DevSummary *sum, int64_t N, int32_t frame)
 {
     __shared__ float smf[32];
-    __shared__ double smd[32][5];
+    __shared__ double smd[32][8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     float m = -INFINITY;
     for (int b = threadIdx.x; b < n; b += blockDim.x)
@@ -226,7 +227,7 @@ __device__ void grad_finalize(const GradPartial *part, int n, DevSummary *sum, i
     float M = -INFINITY;
     for (int w = 0; w < nw; ++w)
         M = fmaxf(M, smf[w]);
-    double acc[5] = {0, 0, 0, 0, 0};
+    double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // s0, s[4] (and three unused)
     for (int b = threadIdx.x; b < n; b += blockDim.x) {
         const float qm = __ldcg(&part[b].m);
         if (qm > -INFINITY) {
@@ -236,28 +237,32 @@ __device__ void grad_finalize(const GradPartial *part, int n, DevSummary *sum, i
                 acc[1 + c] += __ldcg(&part[b].s[c]) * f;
         }
     }
-    for (int c = 0; c < 5; ++c)
-        acc[c] = warp_sum_d(acc[c]);
-    if (lane == 0)
-        for (int c = 0; c < 5; ++c)
-            smd[warp][c] = acc[c];
+    const double r = warp_sum8_d(acc);
+    if ((lane & 3) == 0)
+        smd[warp][lane_value(lane)] = r;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double t[5] = {0, 0, 0, 0, 0};
+    if (warp == 0) {
+        // lane c holds the c-th total; lanes 0 and 7 take one logarithm each
+        double t = 0;
         for (int w = 0; w < nw; ++w)
-            for (int c = 0; c < 5; ++c)
-                t[c] += smd[w][c];
-        const double le = (double)M + log(t[0]) - log((double)N);
-        sum->log_total = (double)M + log(t[0]);
-        sum->log_evidence = le;
-        sum->max_lw = (double)M;
-        sum->M = M;
-        sum->frame = frame;
-        sum->grad_L += le;
-        for (int c = 0; c < 4; ++c)
-            sum->grad_g[c] += t[1 + c] / t[0];
-        if (!(t[0] > 0.0))
-            sum->flags |= FLAG_DEGENERATE;
+            t += smd[w][lane & 7];
+        const double t0 = __shfl_sync(0xffffffffu, t, 0);
+        const double q = t / t0;
+        const double lg = log(lane == 0 ? t0 : (lane == 7 ? (double)N : 1.0));
+        const double ln = __shfl_sync(0xffffffffu, lg, 7);
+        if (lane >= 1 && lane <= 4)
+            sum->grad_g[lane - 1] += q;
+        if (lane == 0) {
+            const double le = (double)M + lg - ln;
+            sum->log_total = (double)M + lg;
+            sum->log_evidence = le;
+            sum->max_lw = (double)M;
+            sum->M = M;
+            sum->frame = frame;
+            sum->grad_L += le;
+            if (!(t0 > 0.0))
+                sum->flags |= FLAG_DEGENERATE;
+        }
     }
 }
 
