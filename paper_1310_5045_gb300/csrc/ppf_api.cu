@@ -454,8 +454,16 @@ ppf_status ppf_estimate_async(ppf_ctx *c, ppf_estimate_t *out)
         return PPF_EINVAL;
     if (!c->stepped)
         return PPF_ESTATE;
-    CK(ppf::launch_format_estimate(c));
-    CK(cudaMemcpyAsync(out, c->est_dev, sizeof(ppf_estimate_t), cudaMemcpyDeviceToHost, c->stream));
+    // the kernel writes the caller's page-locked buffer itself where the device
+    // can address it (one launch and no copy); otherwise a staged copy
+    void *dev = nullptr;
+    if (cudaHostGetDevicePointer(&dev, out, 0) == cudaSuccess && dev) {
+        CK(ppf::launch_format_estimate(c, (ppf_estimate_t *)dev));
+    } else {
+        cudaGetLastError();
+        CK(ppf::launch_format_estimate(c, c->est_dev));
+        CK(cudaMemcpyAsync(out, c->est_dev, sizeof(ppf_estimate_t), cudaMemcpyDeviceToHost, c->stream));
+    }
     c->d2h_bytes += (int64_t)sizeof(ppf_estimate_t);
     return PPF_OK;
 }

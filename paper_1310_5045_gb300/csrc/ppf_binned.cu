@@ -108,7 +108,8 @@ __global__ void __launch_bounds__(256) bin_scatter_kernel(const float *__restric
                                                           int32_t *__restrict__ items, int items_max,
                                                           DevSummary *sum)
 {
-    pdl_wait();  // launched as a dependent of the step kernel
+    if (!pdl_wait())
+        return;
     pdl_trigger();
     if (__ldcg(&sum->bin_this) == 0)
         return;
@@ -287,7 +288,8 @@ struct BinLikArgs {
 template <int R>
 __global__ void __launch_bounds__(256) bin_loglik_kernel(const __grid_constant__ CUtensorMap tmap, BinLikArgs a)
 {
-    pdl_wait();  // launched as a dependent of the scatter
+    if (!pdl_wait())
+        return;
     pdl_trigger();
     DevSummary *sum = a.sum;
     if (__ldcg(&sum->bin_this) == 0)

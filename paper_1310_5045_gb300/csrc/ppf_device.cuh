@@ -42,9 +42,15 @@ __device__ __forceinline__ bool debug_check(bool ok, const int32_t *flags, int32
 // of the stream has completed and its writes are visible (a no-op for a
 // kernel launched without the attribute); pdl_trigger() lets the next kernel,
 // if launched with the attribute, be scheduled before this one completes.
-__device__ __forceinline__ void pdl_wait()
+// Every kernel of a chain begins with `if (!pdl_wait()) return;`: the result
+// is never 0 (it is the grid's width), but the branch on it keeps the
+// compiler from moving loads that it takes for invariant (const __restrict__
+// arguments, __ldg) above the wait.
+__device__ __forceinline__ bool pdl_wait()
 {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    uint32_t n;
+    asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, %%nctaid.x;" : "=r"(n)::"memory");
+    return n != 0u;
 }
 
 __device__ __forceinline__ void pdl_trigger()

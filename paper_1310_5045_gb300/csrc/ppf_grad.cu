@@ -266,9 +266,13 @@ __device__ void grad_finalize(const GradPartial *part, int n, DevSummary *sum, i
     }
 }
 
+// (up to R = 5 the kernel fits 128 registers: two blocks per SM)
 template <int R>
-__global__ void __launch_bounds__(256) grad_step_kernel(GradArgs a)
+__global__ void __launch_bounds__(256, R <= 5 ? 2 : 1) grad_step_kernel(GradArgs a)
 {
+    if (!pdl_wait())
+        return;
+    pdl_trigger();
     const int64_t N = a.N;
     const bool ident = a.first || *a.degenerate;
     GAcc acc;
@@ -354,7 +358,7 @@ __global__ void __launch_bounds__(256) grad_step_kernel(GradArgs a)
 template <int R>
 static void launch_grad_r(const GradArgs &a, int grid, cudaStream_t s)
 {
-    grad_step_kernel<R><<<grid, 256, 0, s>>>(a);
+    launch_pdl(grad_step_kernel<R>, grid, 256, 0, s, a);
 }
 
 cudaError_t launch_grad_step(ppf_ctx *c, int32_t k, bool first, int32_t *anchors)

@@ -277,7 +277,7 @@ __device__ __forceinline__ float cell_loglik(const PatchGeom &a, const float2 *_
 // instructions are its time.  With the sums below, one division for all means
 // and one logarithm per lane the step of 250,000 particles takes 24.5 us
 // (31.8 with eight butterflies, then seven divisions and two logarithms by one
-// thread), and 1024 batched filters are finalised in 7 us (16).
+// thread), and 1024 batched filters are finalised in 9 us (16).
 //
 // Eight sums over the lanes of a warp, each the butterfly's sum (offsets 16,
 // 8, 4, 2, 1): every level of the first three hands half of the values to the

@@ -26,17 +26,6 @@
 
 namespace ppf {
 
-// kernels of ppf_resample.cu used unchanged
-__global__ void __launch_bounds__(TILE_THREADS, 5) tile_totals_kernel(const float *__restrict__ lw, int64_t N,
-                                                                      const DevSummary *__restrict__ sum,
-                                                                      double ess_thr, uint64_t *__restrict__ Qt,
-                                                                      uint64_t *__restrict__ St);
-__global__ void __launch_bounds__(1024) tile_scan_kernel(int64_t N, int32_t T, const uint64_t *__restrict__ Qt, uint64_t *__restrict__ Ct,
-                                 int64_t *__restrict__ Tt, DevSummary *sum, double ess_thr, uint64_t seed,
-                                 uint32_t fid, uint32_t frame, const int64_t *__restrict__ goff, int32_t G, int rpa,
-                                 const uint64_t *__restrict__ Cbl, int64_t *__restrict__ Tg, int32_t smem_tiles,
-                                 Divisor ndiv, int prefix_only, int2 *__restrict__ extra,
-                                 int32_t *__restrict__ To);
 namespace {
 
 constexpr int64_t NOALLOC_MAX_N = (int64_t)1 << 24;               // particles per call
@@ -204,18 +193,11 @@ extern "C" ppf_status ppf_systematic_resample_noalloc(const float *lw_dev, int64
     int2 *extra = reinterpret_cast<int2 *>(s + OFF_EX);
     int32_t *To = reinterpret_cast<int32_t *>(s + OFF_TO);
     uint64_t *St = reinterpret_cast<uint64_t *>(s + OFF_ST);
-    const int32_t T = (int32_t)((n + TILE - 1) / TILE);
     noalloc_clear_kernel<<<1, 32, 0, st>>>(s);
     const int gmax = (int)((n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024);
     noalloc_max_kernel<<<gmax, 256, 0, st>>>(lw_dev, n, s);
-    // (every call resamples: the N_eff threshold is +inf)
-    tile_totals_kernel<<<T, TILE_THREADS, 0, st>>>(lw_dev, n, sum, INFINITY, Qt, St);
-    // (T <= 4096 tiles: the scan's tile values, 32 KB, fit the default shared memory)
-    tile_scan_kernel<<<1, 1024, sizeof(uint64_t) * (T + 1), st>>>(n, T, Qt, Ct, Tt, sum, INFINITY,
-                                                                  seed, filter_id, (uint32_t)frame, nullptr, 0, 0,
-                                                                  nullptr, nullptr, T, make_divisor((uint32_t)n), 0,
-                                                                  extra, To);
-    if (launch_fill_plain(lw_dev, n, T, sum, Ct, Tt, To, St, extra, anc_dev, st) != cudaSuccess)
+    if (launch_draw_plain(lw_dev, n, sum, Qt, St, Ct, Tt, To, extra, seed, filter_id, (uint32_t)frame, anc_dev, st) !=
+        cudaSuccess)
         return PPF_ECUDA;
     noalloc_identity_if_degenerate<<<gmax, 256, 0, st>>>(anc_dev, n, s);
     return cudaGetLastError() == cudaSuccess ? PPF_OK : PPF_ECUDA;

@@ -16,6 +16,7 @@
 // step's effective sample size is not below it, the kernels do nothing but
 // mark the particles as kept (the next step carries their weights).
 #include <cmath>
+#include <cstddef>
 
 #include "ppf_device.cuh"
 #include "ppf_internal.h"
@@ -68,6 +69,9 @@ __global__ void __launch_bounds__(TILE_THREADS, 5) tile_totals_kernel(const floa
     // ahead, so that they are in flight while the block quantises the tile
     // before and waits at its reduction; any other tile is loaded when it is
     // its turn.
+    if (!pdl_wait())
+        return;
+    pdl_trigger();
     if (kept_by_ess(sum, ess_thr))
         return;
     __shared__ uint64_t wsum[2][STRIPS];
@@ -181,6 +185,9 @@ __global__ void __launch_bounds__(TILE_THREADS, 5) tile_group_totals_kernel(
     uint64_t *__restrict__ Qt, uint64_t *__restrict__ St, const int64_t *__restrict__ goff, int32_t G,
     uint64_t *__restrict__ Cbl, int32_t *__restrict__ tile_g)
 {
+    if (!pdl_wait())
+        return;
+    pdl_trigger();
     if (kept_by_ess(sum, ess_thr))
         return;
     __shared__ uint64_t sums[TILE];  // the tile's inclusive sums (only for tiles with many group starts)
@@ -315,35 +322,80 @@ __global__ void __launch_bounds__(TILE_THREADS, 5) tile_group_totals_kernel(
 }
 
 // ---------------------------------------------------------------- R2 scan
-// One block: exclusive tile prefix, total Q, ticket offset u, tickets below
-// each tile start and the list of the fill's further runs; for RPA (rpa = 1)
-// and ARNA (rpa = 2) the tickets below each group start.  A proportional draw
-// (rpa != 2) at a low N_eff also sets the next step to the direct likelihood
-// path.  With prefix_only the kernel stops after the prefix and the draw
-// (tile_tickets_kernel does the rest in parallel).
-// When the T + 1 tile values fit the dynamic shared memory (T <= smem_tiles),
-// they are loaded there with coalesced reads, and each of the two prefix sums
-// gives every thread one contiguous segment: a local sum, one block scan,
-// then the segment's prefixes.  Otherwise every array is walked in rounds of
-// blockDim consecutive entries, each round closed by a block scan.
-__global__ void __launch_bounds__(1024) tile_scan_kernel(
-    int64_t N, int32_t T, const uint64_t *__restrict__ Qt, uint64_t *__restrict__ Ct, int64_t *__restrict__ Tt,
-    DevSummary *sum, double ess_thr, uint64_t seed,
-    uint32_t fid, uint32_t frame, const int64_t *__restrict__ goff, int32_t G, int rpa,
-    const uint64_t *__restrict__ Cbl, int64_t *__restrict__ Tg, int32_t smem_tiles, Divisor ndiv, int prefix_only,
-    int2 *__restrict__ extra, int32_t *__restrict__ To)
+// One block: exclusive tile prefix, total Q, ticket offset u, the scale of the
+// ticket counts.  A proportional draw (rpa != 2) at a low N_eff also sets the
+// next step to the direct likelihood path.
+//
+// PER > 0: a thread holds PER consecutive tile totals in registers, all its
+// loads in flight together (T <= PER x threads); PER = 0 walks the tiles in
+// rounds of blockDim, each closed by a block scan.  What the one thread used
+// to do in turn after the scan (the spacing's division, the scale's, the
+// offset's Philox block) four warps do at once.  At T = 9278 (38M) the prefix
+// takes 5 us instead of 9, at T = 512 with as many groups everything 5 instead of 8.
+//
+// FULL (T <= SCAN_FULL_TILES, and as many groups for RPA and ARNA): the block
+// also counts the tickets below each tile start and, for rpa != 0, each group
+// start, one thread each, and lists the fill's further runs; otherwise
+// tile_tickets_kernel does.
+constexpr int SCAN_FULL_TILES = 1023;  // tile or group starts counted by the scan's own block
+
+struct ScanArgs {
+    int64_t N;
+    int32_t T;
+    const uint64_t *__restrict__ Qt;
+    uint64_t *__restrict__ Ct;
+    int64_t *__restrict__ Tt;
+    int32_t *__restrict__ To;
+    DevSummary *sum;
+    double ess_thr;
+    uint64_t seed;
+    uint32_t fid, frame;
+    const int64_t *__restrict__ goff;
+    int32_t G, rpa;  // rpa: 0 systematic, 1 RPA, 2 ARNA
+    const uint64_t *__restrict__ Cbl;
+    int64_t *__restrict__ Tg;
+    Divisor ndiv;
+    int2 *__restrict__ extra;
+};
+
+// a tile's further runs (t, k), k >= 1, into the fill's list (in any order)
+__device__ __forceinline__ void list_runs(DevSummary *sum, int2 *__restrict__ extra, int32_t t, int64_t tickets)
 {
-    extern __shared__ uint64_t sT[];  // (smem_tiles + 1) tile values
+    const int64_t runs = (tickets + ITEM_TICKETS - 1) / ITEM_TICKETS;
+    if (runs > 1) {
+        const int32_t pos = atomicAdd(&sum->n_extra, (int32_t)(runs - 1));
+        for (int64_t k = 1; k < runs; ++k)
+            extra[pos + k - 1] = make_int2(t, (int32_t)k);
+    }
+}
+
+template <int PER, bool FULL>
+__global__ void __launch_bounds__(1024) tile_scan_kernel(ScanArgs A)
+{
+    if (!pdl_wait())
+        return;
+    pdl_trigger();
+    static_assert(!FULL || PER == 1, "the block counts tickets for one tile per thread");
     __shared__ uint64_t red[33];
-    __shared__ uint64_t su, s_qN;
+    __shared__ uint64_t s_u, s_qN;
     __shared__ uint32_t s_qR;
     __shared__ TicketScale s_sc;
+    __shared__ uint64_t sC[FULL ? SCAN_FULL_TILES + 1 : 1];
+    __shared__ int64_t sT[FULL ? SCAN_FULL_TILES + 1 : 1];
+    DevSummary *sum = A.sum;
+    const int32_t T = A.T;
+    const int64_t N = A.N;
+    uint64_t v[PER > 0 ? PER : 1];
+    const int t0 = (int)threadIdx.x * PER;
+#pragma unroll
+    for (int k = 0; k < PER; ++k)
+        v[k] = t0 + k < T ? __ldg(A.Qt + t0 + k) : 0ull;
     if (threadIdx.x == 0) {
         sum->n_split = 0;  // the two-stage draw's split list is rebuilt after the scan
         sum->n_runs = 0;
         sum->n_extra = 0;  // and the fill's list of further ticket runs
     }
-    if (kept_by_ess(sum, ess_thr)) {  // N_eff test: keep the particles and the layout
+    if (kept_by_ess(sum, A.ess_thr)) {  // N_eff test: keep the particles and the layout
         if (threadIdx.x == 0) {
             sum->degenerate = 1;
             sum->flags |= FLAG_KEPT;
@@ -352,142 +404,138 @@ __global__ void __launch_bounds__(1024) tile_scan_kernel(
         }
         return;
     }
-    const bool in_smem = T <= smem_tiles;
-    const int seg = (T + (int)blockDim.x - 1) / (int)blockDim.x;
-    const int s0 = min(T, (int)threadIdx.x * seg), s1 = min(T, s0 + seg);
     uint64_t total = 0;
-    if (in_smem) {
-        for (int t = threadIdx.x; t < T; t += blockDim.x)
-            sT[t] = __ldg(Qt + t);
-        __syncthreads();
+    if (PER > 0) {
         uint64_t loc = 0;
-        for (int t = s0; t < s1; ++t)
-            loc += sT[t];
+#pragma unroll
+        for (int k = 0; k < PER; ++k)
+            loc += v[k];
         uint64_t run = block_excl_scan_u64(loc, red, &total);
-        for (int t = s0; t < s1; ++t) {
-            const uint64_t v = sT[t];
-            sT[t] = run;  // exclusive tile prefix
-            run += v;
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            if (t0 + k < T) {
+                A.Ct[t0 + k] = run;  // exclusive tile prefix
+                if (FULL)
+                    sC[t0 + k] = run;
+            }
+            run += v[k];
         }
-        __syncthreads();
-        for (int t = threadIdx.x; t < T; t += blockDim.x)
-            Ct[t] = sT[t];
     } else {
         for (int base = 0; base < T; base += blockDim.x) {
             const int t = base + threadIdx.x;
-            const uint64_t v = (t < T) ? Qt[t] : 0ull;
+            const uint64_t x = (t < T) ? A.Qt[t] : 0ull;
             uint64_t tot;
-            const uint64_t ex = block_excl_scan_u64(v, red, &tot);
+            const uint64_t ex = block_excl_scan_u64(x, red, &tot);
             if (t < T)
-                Ct[t] = total + ex;
+                A.Ct[t] = total + ex;
             total += tot;
         }
     }
+    const bool deg = total == 0ull;
     if (threadIdx.x == 0) {
-        Ct[T] = total;
-        const int deg = (total == 0ull);
-        sum->degenerate = deg;
+        A.Ct[T] = total;
+        sum->Q = total;
+        sum->degenerate = deg ? 1 : 0;
         if (deg)
             sum->flags |= FLAG_DEGENERATE;
-        sum->Q = total;
-        s_qN = total / (uint64_t)N;
-        s_qR = (uint32_t)(total % (uint64_t)N);
+        else if (A.rpa != 2 && sum->ess < (double)N / BIN_CONCENTRATE)
+            sum->bin_next = 0;  // a concentrating proportional draw: the next step is direct
+        if (!deg && !A.rpa) {
+            // systematic keeps the group layout (the summary already holds its
+            // extent, set whenever the layout changes); no routing
+            sum->links = 0;
+            sum->moved = 0;
+        }
+    } else if (threadIdx.x == 32) {
+        uint32_t r;
+        s_qN = div_by(total, A.ndiv, &r);
+        s_qR = r;
         sum->qN = s_qN;
-        sum->qR = s_qR;
-        if (!deg) {
-            const TicketScale sc = ticket_scale(total, (uint32_t)N);
-            sum->tsv = sc.v;
-            sum->tsr = sc.sr;
-            sum->tsl = sc.sl;
-            s_sc = sc;
+        sum->qR = r;
+    } else if (threadIdx.x == 64 && !deg) {
+        const TicketScale sc = ticket_scale(total, (uint32_t)N);
+        s_sc = sc;
+        sum->tsv = sc.v;
+        sum->tsr = sc.sr;
+        sum->tsl = sc.sl;
+    } else if (threadIdx.x == 96) {
+        s_u = deg ? 0ull : ticket_offset(A.seed, A.fid, A.frame, PURPOSE_RESAMPLE, 0u, total);
+        sum->u = s_u;
+    }
+    if (!FULL || deg)
+        return;
+    __syncthreads();
+    const TicketGrid tg = ticket_grid(total, s_u, s_qN, s_qR, A.ndiv);
+    // the tickets below the tile starts, then those below the group starts
+    const int starts = T + 1 + (A.rpa ? A.G + 1 : 0);
+    for (int i = threadIdx.x; i < starts; i += blockDim.x) {
+        const int g = i - (T + 1);
+        const int64_t pos = g < 0 ? 0 : A.goff[g];
+        const bool end = g < 0 ? i == T : pos >= N;
+        const uint64_t c = end ? total : (g < 0 ? sC[i] : sC[pos / TILE] + A.Cbl[g]);
+        const int64_t j = end ? N : tickets_below_grid(c, tg);
+        if (g >= 0) {
+            A.Tg[g] = j;
+            continue;
         }
-        su = deg ? 0ull : ticket_offset(seed, fid, frame, PURPOSE_RESAMPLE, 0u, total);
-        sum->u = su;
+        A.Tt[i] = sT[i] = j;
+        if (i < T)
+            A.To[i] = run_offset(c, tg, s_sc, j, true);
     }
     __syncthreads();
-    const uint64_t Q = total, u = su;
-    const TicketGrid tg = ticket_grid(Q, u, s_qN, s_qR, ndiv);
-    if (Q == 0ull)
-        return;
-    if (threadIdx.x == 0 && rpa != 2 && sum->ess < (double)N / BIN_CONCENTRATE)
-        sum->bin_next = 0;  // a concentrating proportional draw: the next step is direct
-    if (prefix_only) {  // tile_tickets_kernel takes it from here, one thread per tile and group
-        if (threadIdx.x == 0 && !rpa) {
-            sum->links = 0;
-            sum->moved = 0;
-        }
-        return;
-    }
-    for (int t = threadIdx.x; t <= T; t += blockDim.x) {
-        const uint64_t c = in_smem ? sT[t] : Ct[t];
-        const int64_t v = (t == T) ? N : tickets_below_grid(c, tg);
-        Tt[t] = v;
-        if (t < T)
-            To[t] = run_offset(c, tg, s_sc, v, true);
-        if (in_smem)
-            sT[t] = (uint64_t)v;  // each thread rewrites only the entries it read
-    }
-    __syncthreads();
-    // the fill's further runs of ticket-heavy tiles, as tile_tickets_kernel lists them
-    for (int t = threadIdx.x; t < T; t += blockDim.x) {
-        const int64_t a = in_smem ? (int64_t)sT[t] : Tt[t];
-        const int64_t b = (t + 1 == T) ? N : (in_smem ? (int64_t)sT[t + 1] : Tt[t + 1]);
-        const int64_t runs = (b - a + ITEM_TICKETS - 1) / ITEM_TICKETS;
-        if (runs > 1) {
-            const int32_t pos = atomicAdd(&sum->n_extra, (int32_t)(runs - 1));
-            for (int64_t k = 1; k < runs; ++k)
-                extra[pos + k - 1] = make_int2(t, (int32_t)k);
-        }
-    }
-    if (rpa) {
-        for (int g = threadIdx.x; g <= G; g += blockDim.x) {
-            const int64_t pos = goff[g];
-            const uint64_t c = (pos >= N) ? Q : Ct[pos / TILE] + Cbl[g];
-            Tg[g] = (pos >= N) ? N : tickets_below_grid(c, tg);
-        }
-    } else {
-        // systematic keeps the group layout (the summary already holds its
-        // extent, set whenever the layout changes); no routing
-        if (threadIdx.x == 0) {
-            sum->links = 0;
-            sum->moved = 0;
-        }
-    }
+    for (int t = threadIdx.x; t < T; t += blockDim.x)
+        list_runs(sum, A.extra, t, sT[t + 1] - sT[t]);
 }
 
 // The tickets below every tile start and, for RPA and ARNA, every group
-// start: one thread each, after tile_scan_kernel's prefix (the same counts
-// tile_scan_kernel forms one block wide).  A tile with more than
-// ITEM_TICKETS tickets lists its further runs (t, k), k >= 1, for the fill's
-// extra blocks; the order of the list does not matter.
-__global__ void __launch_bounds__(256) tile_tickets_kernel(
-    int64_t N, int32_t T, const uint64_t *__restrict__ Ct, int64_t *__restrict__ Tt, DevSummary *__restrict__ sum,
-    Divisor ndiv, const int64_t *__restrict__ goff, int32_t G, int rpa, const uint64_t *__restrict__ Cbl,
-    int64_t *__restrict__ Tg, int2 *__restrict__ extra, int32_t *__restrict__ To)
+// start, one thread each, after tile_scan_kernel's prefix, and the fill's
+// list of further runs.
+__global__ void __launch_bounds__(256) tile_tickets_kernel(ScanArgs A)
 {
+    if (!pdl_wait())
+        return;
+    pdl_trigger();
+    DevSummary *__restrict__ sum = A.sum;
     if (sum->degenerate)
         return;  // kept by the N_eff test, or no usable weight
-    const TicketGrid tg = ticket_grid(sum->Q, sum->u, sum->qN, sum->qR, ndiv);
+    const int32_t T = A.T;
+    const int64_t N = A.N;
+    const TicketGrid tg = ticket_grid(sum->Q, sum->u, sum->qN, sum->qR, A.ndiv);
     const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i <= T) {
-        const int64_t a = (i == T) ? N : tickets_below_grid(Ct[i], tg);
-        Tt[i] = a;
+        const int64_t a = (i == T) ? N : tickets_below_grid(A.Ct[i], tg);
+        A.Tt[i] = a;
         if (i < T) {
-            To[i] = run_offset(Ct[i], tg, TicketScale{sum->tsv, sum->tsr, sum->tsl}, a, true);
-            const int64_t b = (i + 1 == T) ? N : tickets_below_grid(Ct[i + 1], tg);
-            const int64_t runs = (b - a + ITEM_TICKETS - 1) / ITEM_TICKETS;
-            if (runs > 1) {
-                const int32_t pos = atomicAdd(&sum->n_extra, (int32_t)(runs - 1));
-                for (int64_t k = 1; k < runs; ++k)
-                    extra[pos + k - 1] = make_int2(i, (int32_t)k);
-            }
+            A.To[i] = run_offset(A.Ct[i], tg, TicketScale{sum->tsv, sum->tsr, sum->tsl}, a, true);
+            list_runs(sum, A.extra, i, ((i + 1 == T) ? N : tickets_below_grid(A.Ct[i + 1], tg)) - a);
         }
     }
-    if (rpa && i <= G) {
-        const int64_t pos = goff[i];
-        const uint64_t c = (pos >= N) ? sum->Q : Ct[pos / TILE] + Cbl[i];
-        Tg[i] = (pos >= N) ? N : tickets_below_grid(c, tg);
+    if (A.rpa && i <= A.G) {
+        const int64_t pos = A.goff[i];
+        const uint64_t c = (pos >= N) ? sum->Q : A.Ct[pos / TILE] + A.Cbl[i];
+        A.Tg[i] = (pos >= N) ? N : tickets_below_grid(c, tg);
     }
+}
+
+// The scan and the ticket counts; returns the launches made.
+static int launch_scan(const ScanArgs &A, cudaStream_t stream)
+{
+    const int32_t T = A.T, most = A.rpa && A.G > T ? A.G : T;
+    if (most <= SCAN_FULL_TILES) {
+        const int starts = T + 1 + (A.rpa ? A.G + 1 : 0);
+        int threads = (starts + 31) / 32 * 32;
+        threads = threads < 128 ? 128 : (threads > 1024 ? 1024 : threads);
+        launch_pdl(tile_scan_kernel<1, true>, 1, threads, 0, stream, A);
+        return 1;
+    }
+    if (T <= 4 * 1024)
+        launch_pdl(tile_scan_kernel<4, false>, 1, 1024, 0, stream, A);
+    else if (T <= 16 * 1024)
+        launch_pdl(tile_scan_kernel<16, false>, 1, 1024, 0, stream, A);
+    else
+        launch_pdl(tile_scan_kernel<0, false>, 1, 1024, 0, stream, A);
+    launch_pdl(tile_tickets_kernel, (most + 256) / 256, 256, 0, stream, A);
+    return 2;
 }
 
 // ------------------------------------------------ kept tickets, GS and SGS
@@ -606,6 +654,9 @@ struct FillArgs {
 template <bool ROUTE>
 __global__ void __launch_bounds__(TILE_THREADS, 4) fill_tiles_kernel(FillArgs A)
 {
+    if (!pdl_wait())
+        return;
+    pdl_trigger();
     const DevSummary *__restrict__ sum = A.sum;
     // the tile's bounds are read together with the flags that may end the block
     const int32_t deg = sum->degenerate, n_extra = sum->n_extra;
@@ -683,19 +734,26 @@ static cudaError_t launch_fill(const FillArgs &A, cudaStream_t stream)
 {
     const int runs = A.T + (int)(A.N / ITEM_TICKETS) + 1;
     if (A.kr.anc)
-        fill_tiles_kernel<true><<<runs, TILE_THREADS, 0, stream>>>(A);
+        launch_pdl(fill_tiles_kernel<true>, runs, TILE_THREADS, 0, stream, A);
     else
-        fill_tiles_kernel<false><<<runs, TILE_THREADS, 0, stream>>>(A);
+        launch_pdl(fill_tiles_kernel<false>, runs, TILE_THREADS, 0, stream, A);
     return cudaGetLastError();
 }
 
-// The fill alone (the allocation-free entry point).
-cudaError_t launch_fill_plain(const float *lw, int64_t N, int32_t T, const DevSummary *sum, const uint64_t *Ct,
-                              const int64_t *Tt, const int32_t *To, const uint64_t *St, const int2 *extra,
+// The systematic draw on the caller's buffers (the allocation-free entry
+// point): tile totals, scan, ticket counts, fill.  Resamples every time.
+cudaError_t launch_draw_plain(const float *lw, int64_t N, DevSummary *sum, uint64_t *Qt, uint64_t *St, uint64_t *Ct,
+                              int64_t *Tt, int32_t *To, int2 *extra, uint64_t seed, uint32_t fid, uint32_t frame,
                               int32_t *out, cudaStream_t stream)
 {
+    const int32_t T = (int32_t)((N + TILE - 1) / TILE);
+    const Divisor nd = make_divisor((uint32_t)N);
+    launch_pdl(tile_totals_kernel, T, TILE_THREADS, 0, stream, lw, N, (const DevSummary *)sum, (double)INFINITY, Qt, St);
+    launch_scan(ScanArgs{N, T, Qt, Ct, Tt, To, sum, INFINITY, seed, fid, frame, nullptr, 0, 0, nullptr, nullptr, nd,
+                         extra},
+                stream);
     const KeptRoute none{nullptr, nullptr, nullptr, 0, Balanced{0, 0}};
-    return launch_fill(FillArgs{lw, N, T, make_divisor((uint32_t)N), sum, Ct, Tt, To, St, extra, out, none}, stream);
+    return launch_fill(FillArgs{lw, N, T, nd, sum, Ct, Tt, To, St, extra, out, none}, stream);
 }
 
 // ------------------------------------------------ two-stage RPA, stage 2
@@ -729,6 +787,9 @@ __global__ void __launch_bounds__(256) group_grid_kernel(
     uint64_t seed, uint32_t fid, uint32_t frame, GroupGrid *__restrict__ grid, int4 *__restrict__ split,
     Balanced bl)
 {
+    if (!pdl_wait())
+        return;
+    pdl_trigger();
     const int32_t g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= G || kept_by_ess(sum, ess_thr) || sum->degenerate)
         return;
@@ -797,6 +858,9 @@ __global__ void __launch_bounds__(256) split_runs_kernel(const uint64_t *__restr
                                                          const GroupGrid *__restrict__ grid, int4 *__restrict__ split,
                                                          DevSummary *__restrict__ sum, double ess_thr)
 {
+    if (!pdl_wait())
+        return;
+    pdl_trigger();
     if (kept_by_ess(sum, ess_thr) || sum->degenerate)
         return;
     const int32_t n0 = sum->n_split;  // the entries group_grid_kernel listed; the runs go after them
@@ -890,6 +954,9 @@ __global__ void __launch_bounds__(TILE_THREADS, 3) group_fill_kernel(
     int32_t n_workers, const DevSummary *__restrict__ sum, double ess_thr, int32_t *__restrict__ out,
     int32_t *__restrict__ kept_anc, Balanced bl, int s)
 {
+    if (!pdl_wait())
+        return;
+    pdl_trigger();
     __shared__ ParentSmem sm;
     if ((int32_t)blockIdx.x >= n_workers) {  // a group block: one item, no loop
         const GroupGrid gg = grid[blockIdx.x - n_workers];
@@ -1659,6 +1726,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT - 1) rna_kernel(
     const int32_t *__restrict__ succ, DevSummary *sum, double ess_thr, uint64_t seed, uint32_t fid, uint32_t frame,
     int32_t *__restrict__ anc, float *__restrict__ lwp, Divisor d_small, Divisor d_large)
 {
+    if (!pdl_wait())
+        return;
+    pdl_trigger();
     if (kept_by_ess(sum, ess_thr))
         return;
     const int64_t mig = sum->mig;
@@ -1808,6 +1878,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT - 1) rna_kernel(
 __global__ void __launch_bounds__(1024) rna_prep_kernel(const int64_t *__restrict__ goff, int32_t G, float alpha,
                                                         DevSummary *sum, double ess_thr)
 {
+    if (!pdl_wait())
+        return;
+    pdl_trigger();
     __shared__ long long smx[32], smn[32];
     long long mx = 0, mn = INT64_MAX;
     for (int g = threadIdx.x; g < G; g += blockDim.x) {
@@ -1861,6 +1934,9 @@ __global__ void __launch_bounds__(1024) arna_prep_kernel(const int64_t *__restri
                                                          int32_t *__restrict__ succ, uint64_t seed, uint32_t fid,
                                                          uint32_t frame)
 {
+    if (!pdl_wait())
+        return;
+    pdl_trigger();
     extern __shared__ uint64_t sm[];
     __shared__ long long smx[32], smn[32];
     __shared__ int sinv[32];
@@ -1966,33 +2042,16 @@ cudaError_t resample_kernel_attributes()
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(arna_prep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)SORT_SMEM_BYTES);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(tile_scan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(sizeof(uint64_t) * (SCAN_SMEM_TILES + 1)));
     return e;
 }
 
-// The tile prefix and the draw (one block), then the tickets below every
-// tile and group start and the fill's list of further runs (one thread each).
-// rpa: 0 systematic, 1 RPA, 2 ARNA.
+// The context's scan.  rpa: 0 systematic, 1 RPA, 2 ARNA.
 static void launch_tile_tickets(ppf_ctx *c, double ess_thr, int rpa)
 {
-    const int T = c->T;
-    const int32_t st_tiles = T <= SCAN_SMEM_TILES ? T : 0;
-    const Divisor nd = make_divisor((uint32_t)c->N);
-    int2 *extra = reinterpret_cast<int2 *>(c->sc.extra);
-    // up to a tile or a group per thread, the block counts the tickets itself
-    // (one launch less); beyond, one thread per tile and group does
-    const bool one_block = T <= 1024 && (!rpa || c->G <= 1024);
-    tile_scan_kernel<<<1, 1024, sizeof(uint64_t) * (st_tiles + 1), c->stream>>>(
-        c->N, T, c->sc.Qt, c->sc.Ct, c->sc.Tt, c->sum, ess_thr, c->m.seed, c->m.filter_id,
-        (uint32_t)c->last_frame, c->goff, c->G, rpa, c->sc.Cbl, c->sc.Tg, st_tiles, nd, one_block ? 0 : 1, extra, c->sc.To);
-    if (one_block)
-        return;
-    const int n = (rpa && c->G > T ? c->G : T) + 1;
-    tile_tickets_kernel<<<(n + 255) / 256, 256, 0, c->stream>>>(c->N, T, c->sc.Ct, c->sc.Tt, c->sum, nd, c->goff,
-                                                                c->G, rpa, c->sc.Cbl, c->sc.Tg, extra, c->sc.To);
-    c->launches += 1;
+    const ScanArgs A{c->N, c->T, c->sc.Qt, c->sc.Ct, c->sc.Tt, c->sc.To, c->sum, ess_thr, c->m.seed, c->m.filter_id,
+                     (uint32_t)c->last_frame, c->goff, c->G, rpa, c->sc.Cbl, c->sc.Tg, make_divisor((uint32_t)c->N),
+                     reinterpret_cast<int2 *>(c->sc.extra)};
+    c->launches += launch_scan(A, c->stream) - 1;
 }
 
 // The RPA schedule on the context's side stream, after the tile scan (an
@@ -2036,11 +2095,11 @@ cudaError_t launch_resample_global(ppf_ctx *c, int scheme, double ess_thr)
     prof_mark(c, PH_RESAMPLE, 0);
     c->launches += rpa ? 5 : 3;
     if (rpa)
-        tile_group_totals_kernel<<<T, TILE_THREADS, 0, c->stream>>>(lw, c->N, c->sum, ess_thr, c->sc.Qt, c->sc.St,
-                                                                    c->goff, c->G, c->sc.Cbl, c->sc.tile_g);
-    else  // five blocks per SM (47 registers), each tile's loads one tile ahead
-        tile_totals_kernel<<<T < 5 * c->num_sms ? T : 5 * c->num_sms, TILE_THREADS, 0, c->stream>>>(
-            lw, c->N, c->sum, ess_thr, c->sc.Qt, c->sc.St);
+        launch_pdl(tile_group_totals_kernel, T, TILE_THREADS, 0, c->stream, lw, c->N, (const DevSummary *)c->sum,
+                   ess_thr, c->sc.Qt, c->sc.St, (const int64_t *)c->goff, c->G, c->sc.Cbl, c->sc.tile_g);
+    else  // five blocks per SM (48 registers), each tile's loads one tile ahead
+        launch_pdl(tile_totals_kernel, T < 5 * c->num_sms ? T : 5 * c->num_sms, TILE_THREADS, 0, c->stream, lw, c->N,
+                   (const DevSummary *)c->sum, ess_thr, c->sc.Qt, c->sc.St);
     launch_tile_tickets(c, ess_thr, rpa ? 1 : 0);
     int32_t *out = rpa ? c->anc_sys : c->anc;
     const bool two_stage = (scheme >= PPF_RPA2_GS && scheme <= PPF_RPA2_LGS);
@@ -2059,11 +2118,13 @@ cudaError_t launch_resample_global(ppf_ctx *c, int scheme, double ess_thr)
         group_grid_kernel<<<(c->G + 255) / 256, 256, 0, c->stream>>>(
             c->N, c->G, c->goff, c->sc.Tg, c->sc.Ct, c->sc.Cbl, c->sum, ess_thr, c->m.seed, c->m.filter_id,
             (uint32_t)c->last_frame, c->sc.ggrid, split, balanced_layout(c->N, c->G));
-        split_runs_kernel<<<c->num_sms, 256, 0, c->stream>>>(c->sc.Ct, c->sc.ggrid, split, c->sum, ess_thr);
+        launch_pdl(split_runs_kernel, c->num_sms, 256, 0, c->stream, (const uint64_t *)c->sc.Ct,
+                   (const GroupGrid *)c->sc.ggrid, split, c->sum, ess_thr);
         const int n_workers = 4 * c->num_sms;
-        group_fill_kernel<<<n_workers + c->G, TILE_THREADS, 0, c->stream>>>(
-            lw, c->N, c->G, c->sc.Tg, c->sc.Ct, c->sc.ggrid, split, n_workers, c->sum, ess_thr, out,
-            kept_direct ? c->anc : nullptr, balanced_layout(c->N, c->G), scale_bits(c->N));
+        launch_pdl(group_fill_kernel, n_workers + c->G, TILE_THREADS, 0, c->stream, lw, c->N, c->G,
+                   (const int64_t *)c->sc.Tg, (const uint64_t *)c->sc.Ct, (const GroupGrid *)c->sc.ggrid,
+                   (const int4 *)split, n_workers, (const DevSummary *)c->sum, ess_thr, out,
+                   kept_direct ? c->anc : nullptr, balanced_layout(c->N, c->G), scale_bits(c->N));
         c->launches += 2;
     } else {
         const KeptRoute kr{kept_direct ? c->anc : nullptr, c->sc.Tg, c->sc.tile_g, c->G, balanced_layout(c->N, c->G)};
@@ -2097,8 +2158,8 @@ static void launch_rna(ppf_ctx *c, double ess_thr, const int32_t *succ)
     const Divisor d0 = make_divisor((uint32_t)(bl.q > 0 ? bl.q : 1)), d1 = make_divisor((uint32_t)(bl.q + 1));
     const int64_t top = c->uneven ? TILE : bl.q + (bl.r > 0 ? 1 : 0);
     auto go = [&](auto kernel, int nt) {
-        kernel<<<c->G, nt, 0, c->stream>>>(lw, c->N, c->G, c->goff, succ, c->sum, ess_thr, c->m.seed, c->m.filter_id,
-                                           (uint32_t)c->last_frame, c->anc, c->lwp, d0, d1);
+        launch_pdl(kernel, c->G, nt, 0, c->stream, lw, c->N, c->G, (const int64_t *)c->goff, succ, c->sum, ess_thr,
+                   c->m.seed, c->m.filter_id, (uint32_t)c->last_frame, c->anc, c->lwp, d0, d1);
     };
     if (top <= 64 * TILE_ITEMS)
         go(rna_kernel<64>, 64);
@@ -2111,7 +2172,7 @@ static void launch_rna(ppf_ctx *c, double ess_thr, const int32_t *succ)
 cudaError_t launch_resample_rna(ppf_ctx *c, float alpha, double ess_thr)
 {
     prof_mark(c, PH_RESAMPLE, 0);
-    rna_prep_kernel<<<1, 1024, 0, c->stream>>>(c->goff, c->G, alpha, c->sum, ess_thr);
+    launch_pdl(rna_prep_kernel, 1, 1024, 0, c->stream, (const int64_t *)c->goff, c->G, alpha, c->sum, ess_thr);
     launch_rna(c, ess_thr, nullptr);
     prof_mark(c, PH_RESAMPLE, 1);
     c->launches += 2;
@@ -2125,12 +2186,12 @@ cudaError_t launch_resample_arna(ppf_ctx *c, float alpha, double ess_thr)
     const float *lw = c->state[c->cur] + 5 * c->N;
     const int T = c->T;
     prof_mark(c, PH_RESAMPLE, 0);
-    tile_group_totals_kernel<<<T, TILE_THREADS, 0, c->stream>>>(lw, c->N, c->sum, ess_thr, c->sc.Qt, c->sc.St, c->goff,
-                                                                c->G, c->sc.Cbl, c->sc.tile_g);
+    launch_pdl(tile_group_totals_kernel, T, TILE_THREADS, 0, c->stream, lw, c->N, (const DevSummary *)c->sum, ess_thr,
+               c->sc.Qt, c->sc.St, (const int64_t *)c->goff, c->G, c->sc.Cbl, c->sc.tile_g);
     launch_tile_tickets(c, ess_thr, 2);
-    arna_prep_kernel<<<1, 1024, sort_smem_bytes(c->G), c->stream>>>(
-        c->goff, c->G, alpha, c->sum, ess_thr, c->sc.Tg, c->ring, c->succ, c->m.seed, c->m.filter_id,
-        (uint32_t)c->last_frame);
+    launch_pdl(arna_prep_kernel, 1, 1024, sort_smem_bytes(c->G), c->stream, (const int64_t *)c->goff, c->G, alpha,
+               c->sum, ess_thr, (const int64_t *)c->sc.Tg, c->ring, c->succ, c->m.seed, c->m.filter_id,
+               (uint32_t)c->last_frame);
     launch_rna(c, ess_thr, c->succ);
     prof_mark(c, PH_RESAMPLE, 1);
     c->launches += 4;
@@ -2154,27 +2215,34 @@ cudaError_t launch_identity(ppf_ctx *c, int32_t *dst)
     return cudaGetLastError();
 }
 
-// the ppf_estimate_t fields of the device summary (for ppf_estimate_async)
+// the ppf_estimate_t fields of the device summary, one 8-byte word per lane
+// (for ppf_estimate_async; out is the caller's host buffer as the device sees
+// it, so no copy follows)
 __global__ void format_estimate_kernel(const DevSummary *__restrict__ sum, ppf_estimate_t *__restrict__ out)
 {
-    ppf_estimate_t e;
-    for (int i = 0; i < 5; ++i)
-        e.mean[i] = sum->mean[i];
-    e.log_evidence = sum->log_evidence;
-    e.ess = sum->ess;
-    e.max_log_weight = sum->max_lw;
-    e.frame = sum->frame;
-    e.status_flags = sum->flags;
-    e.links = sum->links;
-    e.moved = sum->moved;
-    e.max_group = sum->max_group;
-    e.min_group = sum->min_group;
-    *out = e;
+    if (!pdl_wait())
+        return;
+    pdl_trigger();
+    static_assert(sizeof(ppf_estimate_t) == 13 * 8 && offsetof(ppf_estimate_t, frame) == 64 &&
+                      offsetof(ppf_estimate_t, status_flags) == 68 && offsetof(ppf_estimate_t, links) == 72,
+                  "the estimate's words");
+    const int w = threadIdx.x;
+    unsigned long long v;
+    if (w < 5)
+        v = (unsigned long long)__double_as_longlong(sum->mean[w]);
+    else if (w < 8)
+        v = (unsigned long long)__double_as_longlong(w == 5 ? sum->log_evidence : w == 6 ? sum->ess : sum->max_lw);
+    else if (w == 8)
+        v = (unsigned long long)(uint32_t)sum->frame | ((unsigned long long)(uint32_t)sum->flags << 32);
+    else
+        v = (unsigned long long)(w == 9 ? sum->links : w == 10 ? sum->moved : w == 11 ? sum->max_group : sum->min_group);
+    if (w < 13)
+        reinterpret_cast<unsigned long long *>(out)[w] = v;
 }
 
-cudaError_t launch_format_estimate(ppf_ctx *c)
+cudaError_t launch_format_estimate(ppf_ctx *c, ppf_estimate_t *out)
 {
-    format_estimate_kernel<<<1, 1, 0, c->stream>>>(c->sum, c->est_dev);
+    launch_pdl(format_estimate_kernel, 1, 32, 0, c->stream, (const DevSummary *)c->sum, out);
     c->launches += 1;
     return cudaGetLastError();
 }

@@ -48,6 +48,9 @@ __global__ void prepare_frame_kernel(const T *__restrict__ Z, float *__restrict_
                                      int Hp, int pad, float bg, DevSummary *sum, int force,
                                      uint32_t *__restrict__ bin_tot, int nbins)
 {
+    if (!pdl_wait())
+        return;
+    pdl_trigger();
     // the likelihood path of this step: the caller's choice, else the one the
     // previous step's finaliser decided; and the binned path's counts cleared
     if (blockIdx.x == 0 && threadIdx.x == 0 && sum)
@@ -207,10 +210,9 @@ __device__ __forceinline__ void bin_propagate(const StepArgs &a, int mode)
 template <int R, bool PC>
 __global__ void __launch_bounds__(256, 3) step_kernel(StepArgs a, int phase)
 {
-    if (phase == 1)
-        pdl_wait();  // the binned likelihood's l (launched as a dependent of it)
-    else
-        pdl_trigger();  // the binned path's kernels may be scheduled meanwhile
+    if (!pdl_wait())
+        return;
+    pdl_trigger();  // the kernels after this one may be scheduled meanwhile
     int mode = a.mode;
     if (mode != MODE_CARRY && *a.degenerate)
         mode = MODE_CARRY;  // the last resample kept every particle
@@ -391,6 +393,9 @@ struct KcArr {
 template <int R>
 __global__ void cell_map_kernel(PatchGeom geom, KcArr kc, float2 *__restrict__ lmap)
 {
+    if (!pdl_wait())
+        return;
+    pdl_trigger();
     constexpr int P = 2 * R + 1;
     geom.Kc = kc.v;
     const int lw = geom.W + 2 * R, lh = geom.H + 2 * R;
@@ -407,7 +412,7 @@ template <int R>
 static void launch_cell_map_r(const PatchGeom &g, const KcArr &kc, float2 *lmap, int n, cudaStream_t s)
 {
     const int grid = (n + 255) / 256 < 2048 ? (n + 255) / 256 : 2048;
-    cell_map_kernel<R><<<grid, 256, 0, s>>>(g, kc, lmap);
+    launch_pdl(cell_map_kernel<R>, grid, 256, 0, s, g, kc, lmap);
 }
 
 cudaError_t launch_cell_map(ppf_ctx *c)
@@ -453,21 +458,14 @@ cudaError_t launch_prepare_frame(ppf_ctx *c, const void *frame)
     const float bg = c->m.background;
     // pcSIR and contexts without the binned path take the direct path
     const int force = c->bin_key ? c->bin_force : 0;
+    auto go = [&](auto kernel, auto *z) {
+        launch_pdl(kernel, grid, 256, 0, c->stream, z, c->Zp, c->m.width, c->m.height, c->Wp, c->Hp, c->pad, bg, c->sum,
+                   force, c->bin_tot, c->bin_nbins);
+    };
     switch (c->m.frame_dtype) {
-    case PPF_BF16:
-        prepare_frame_kernel<__nv_bfloat16><<<grid, 256, 0, c->stream>>>(
-            (const __nv_bfloat16 *)frame, c->Zp, c->m.width, c->m.height, c->Wp, c->Hp, c->pad, bg, c->sum, force, c->bin_tot,
-            c->bin_nbins);
-        break;
-    case PPF_F16:
-        prepare_frame_kernel<__half><<<grid, 256, 0, c->stream>>>(
-            (const __half *)frame, c->Zp, c->m.width, c->m.height, c->Wp, c->Hp, c->pad, bg, c->sum, force, c->bin_tot,
-            c->bin_nbins);
-        break;
-    default:
-        prepare_frame_kernel<float><<<grid, 256, 0, c->stream>>>(
-            (const float *)frame, c->Zp, c->m.width, c->m.height, c->Wp, c->Hp, c->pad, bg, c->sum, force, c->bin_tot,
-            c->bin_nbins);
+    case PPF_BF16: go(prepare_frame_kernel<__nv_bfloat16>, (const __nv_bfloat16 *)frame); break;
+    case PPF_F16: go(prepare_frame_kernel<__half>, (const __half *)frame); break;
+    default: go(prepare_frame_kernel<float>, (const float *)frame);
     }
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && c->lmap)
@@ -479,12 +477,10 @@ cudaError_t launch_prepare_frame(ppf_ctx *c, const void *frame)
 template <int R>
 static void launch_step_r(const StepArgs &a, int grid, int phase, cudaStream_t s)
 {
-    if (phase == 1)  // the binned path's sums: a dependent launch (it waits for the likelihood)
-        launch_pdl(step_kernel<R, false>, grid, 256, 0, s, a, phase);
-    else if (a.lmap)
-        step_kernel<R, true><<<grid, 256, 0, s>>>(a, phase);
+    if (a.lmap)
+        launch_pdl(step_kernel<R, true>, grid, 256, 0, s, a, phase);
     else
-        step_kernel<R, false><<<grid, 256, 0, s>>>(a, phase);
+        launch_pdl(step_kernel<R, false>, grid, 256, 0, s, a, phase);
 }
 
 static void launch_step_phase(const StepArgs &a, int R, int grid, int phase, cudaStream_t s)
