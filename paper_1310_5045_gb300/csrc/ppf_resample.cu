@@ -619,6 +619,201 @@ struct EmitRouted {
     }
 };
 
+// ------------------------------------------- the GS and SGS links, in a block
+// What the RPA schedules read and write (see the RPA schedule below).
+struct SchedArgs {
+    int64_t N;
+    int32_t G;
+    int scheme;
+    const int64_t *goff;
+    int64_t *goff_new;
+    const int64_t *Tg;
+    uint64_t *key;      // [2 * G]  (sender keys, receiver keys)
+    int64_t *val;       // [5 * G]  (PS, PR, sent, recv, merge buffer)
+    int32_t *seg_chunk; // [2G + 2]
+    int64_t *seg_tick, *seg_dst, *seg_len;  // [2G + 1]
+    DevSummary *sum;
+    int links_only;  // the fill wrote the kept segments already: copy work items for the links only
+    Balanced bl;     // the balanced targets n_g
+};
+
+// first index in sorted a[0..n) with a[i] > v
+__device__ __forceinline__ int upper_bound_i32(const int32_t *a, int n, int32_t v)
+{
+    int lo = 0, hi = n;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (a[mid] > v)
+            hi = mid;
+        else
+            lo = mid + 1;
+    }
+    return lo;
+}
+
+// Up to this many groups the GS and SGS schedule runs in the fill's own first
+// block (their fills write the kept tickets, so only the links are left): its
+// lists fit 33 KB next to the fill's buffers at four blocks per SM, and it
+// needs no second stream, events or launch.  By itself the one-block schedule
+// of a side stream took 33 us at 8 groups and 80 us at 1954, most of it a
+// register sort that every thread ran whatever the count and global round
+// trips; a fill of 8M particles takes 30 us.
+constexpr int SCHED_SMALL = 2048;
+
+__host__ __device__ inline int pow2_at_least(int n)
+{
+    int p = 64;
+    while (p < n)
+        p *= 2;
+    return p;
+}
+
+inline size_t sched_small_bytes(int32_t G)
+{
+    return sizeof(uint64_t) * pow2_at_least(G) + sizeof(int32_t) * (2 * (size_t)G + 4);
+}
+
+// The links of GS and SGS: the senders' and receivers' amounts in list order
+// (group order for GS; for SGS by amount, descending, ties by group) are
+// pieces of [0, D), and every distinct piece start begins a link.  All starts
+// of senders are links; a receiver's is one unless a sender starts there too.
+// Output: the balanced offsets and one routing segment per sender and
+// receiver (empty where its start is no link) with its copy work items.
+// Called by every thread of one block; mem: sched_small_bytes(G).
+__device__ void schedule_small(const SchedArgs &A, unsigned char *mem)
+{
+    __shared__ uint64_t red[33];
+    const int32_t G = A.G;
+    const Balanced &bl = A.bl;
+    DevSummary *sum = A.sum;
+    if (sum->degenerate) {
+        for (int g = threadIdx.x; g <= G; g += blockDim.x)
+            A.goff_new[g] = A.goff[g];
+        if (threadIdx.x == 0) {
+            sum->n_chunks = 0;
+            sum->links = 0;
+            sum->moved = 0;
+        }
+        return;
+    }
+    // key: class (receivers above), descending amount, group
+    uint64_t *key = reinterpret_cast<uint64_t *>(mem);
+    int32_t *tg = reinterpret_cast<int32_t *>(key + pow2_at_least(G));
+    int32_t *P = tg + G + 1;  // prefix sums: the senders' and D, then the receivers' and D
+    auto amount = [](uint64_t k) -> int32_t { return 0x7FFFFFFF - (int32_t)((k >> 32) & 0x7FFFFFFFu); };
+    auto group = [](uint64_t k) -> int32_t { return (int32_t)(k & 0xFFFFu); };
+    for (int g = threadIdx.x; g <= G; g += blockDim.x) {
+        tg[g] = (int32_t)A.Tg[g];
+        A.goff_new[g] = balanced_offset(bl, g);
+    }
+    __syncthreads();
+    int nS, nR;
+    {
+        const int per = (G + (int)blockDim.x - 1) / (int)blockDim.x, g0 = (int)threadIdx.x * per;
+        uint64_t c = 0;
+        for (int g = g0; g < g0 + per && g < G; ++g) {
+            const int32_t d = tg[g + 1] - tg[g] - (int32_t)target_of(bl, g);
+            c += d > 0 ? 1ull : (d < 0 ? 1ull << 32 : 0ull);
+        }
+        uint64_t total;
+        const uint64_t at = block_excl_scan_u64(c, red, &total);
+        nS = (int)(uint32_t)total;
+        nR = (int)(total >> 32);
+        int ps = (int)(uint32_t)at, pr = nS + (int)(at >> 32);
+        for (int g = g0; g < g0 + per && g < G; ++g) {
+            const int32_t d = tg[g + 1] - tg[g] - (int32_t)target_of(bl, g);
+            if (d > 0)
+                key[ps++] = ((uint64_t)(uint32_t)(0x7FFFFFFF - d) << 32) | (uint64_t)g;
+            else if (d < 0)
+                key[pr++] = (1ull << 63) | ((uint64_t)(uint32_t)(0x7FFFFFFF + d) << 32) | (uint64_t)g;
+        }
+    }
+    const int n = nS + nR;
+    if (A.scheme != PPF_RPA_GS) {
+        // bitonic sort in shared memory, one pair per thread and round; steps
+        // within 64 keys stay within a warp
+        const int n2 = pow2_at_least(n);
+        for (int i = n + threadIdx.x; i < n2; i += blockDim.x)
+            key[i] = ~0ull;
+        __syncthreads();
+        for (int k = 2; k <= n2; k *= 2)
+            for (int j = k / 2; j > 0; j /= 2) {
+                for (int p = threadIdx.x; p < n2 / 2; p += blockDim.x) {
+                    const int i = 2 * p - (p & (j - 1));
+                    const uint64_t x = key[i], y = key[i + j];
+                    if ((x > y) == ((i & k) == 0)) {
+                        key[i] = y;
+                        key[i + j] = x;
+                    }
+                }
+                if (j >= 64 || (j == 1 && k >= 64))
+                    __syncthreads();
+                else if (j > 32)
+                    __syncthreads();
+                else
+                    __syncwarp();
+            }
+    }
+    __syncthreads();
+    const int per = (n + (int)blockDim.x - 1) / (int)blockDim.x;
+    const int i0 = (int)threadIdx.x * per, i1 = i0 + per < n ? i0 + per : n;
+    int32_t D;
+    {
+        uint64_t s = 0, total;
+        for (int i = i0; i < i1; ++i)
+            s += (uint64_t)(uint32_t)amount(key[i]);
+        uint64_t run = block_excl_scan_u64(s, red, &total);
+        D = (int32_t)(total / 2);  // what the senders give is what the receivers take
+        for (int i = i0; i < i1; ++i) {
+            P[i < nS ? i : i + 1] = (int32_t)(i < nS ? run : run - (uint64_t)D);
+            run += (uint64_t)(uint32_t)amount(key[i]);
+        }
+        if (threadIdx.x == 0)
+            P[nS] = P[n + 1] = D;
+    }
+    __syncthreads();
+    const int32_t *PS = P, *PR = P + nS + 1;
+    uint64_t c = 0;  // links above, copy work items below
+    for (int i = i0; i < i1; ++i) {
+        int si, rj;
+        int32_t a;
+        bool link = true;
+        if (i < nS) {
+            si = i;
+            a = PS[i];
+            rj = upper_bound_i32(PR, nR, a) - 1;
+        } else {
+            rj = i - nS;
+            a = PR[rj];
+            si = upper_bound_i32(PS, nS, a) - 1;
+            link = PS[si] != a;
+        }
+        const int32_t e = PS[si + 1] < PR[rj + 1] ? PS[si + 1] : PR[rj + 1];
+        const int32_t gs = group(key[si]), gr = group(key[nS + rj]);
+        // a sender keeps n_s; a receiver keeps its o_r and is filled after them
+        A.seg_tick[i] = tg[gs] + target_of(bl, gs) + (a - PS[si]);
+        A.seg_dst[i] = balanced_offset(bl, gr) + (tg[gr + 1] - tg[gr]) + (a - PR[rj]);
+        A.seg_len[i] = link ? e - a : 0;
+        if (link)
+            c += (1ull << 32) + (uint64_t)((e - a + COPY_CHUNK - 1) / COPY_CHUNK);
+    }
+    uint64_t total;
+    uint32_t run = (uint32_t)block_excl_scan_u64(c, red, &total);
+    for (int i = i0; i < i1; ++i) {
+        A.seg_chunk[i] = (int32_t)run;
+        run += (uint32_t)((A.seg_len[i] + COPY_CHUNK - 1) / COPY_CHUNK);
+    }
+    if (threadIdx.x == 0) {
+        A.seg_chunk[n] = (int32_t)(uint32_t)total;
+        A.seg_chunk[2 * G + 1] = n;  // the segment count
+        sum->n_chunks = (int32_t)(uint32_t)total;
+        sum->links = (int64_t)(total >> 32);
+        sum->moved = D;
+        sum->max_group = bl.q + (bl.r > 0 ? 1 : 0);
+        sum->min_group = bl.q;
+    }
+}
+
 // ---------------------------------------------------------------- R3 fill
 // Block t < T takes tile t's first ITEM_TICKETS tickets, block T + e the e-th
 // entry (t, k) of the list of further runs; a tile without tickets ends its
@@ -649,6 +844,8 @@ struct FillArgs {
     const int2 *__restrict__ extra;
     int32_t *__restrict__ out;
     KeptRoute kr;
+    int sched;      // the first block runs the schedule
+    SchedArgs sa;
 };
 
 template <bool ROUTE>
@@ -661,6 +858,14 @@ __global__ void __launch_bounds__(TILE_THREADS, 4) fill_tiles_kernel(FillArgs A)
     // the tile's bounds are read together with the flags that may end the block
     const int32_t deg = sum->degenerate, n_extra = sum->n_extra;
     int32_t t = blockIdx.x, k = 0;
+    if (ROUTE && A.sched) {
+        if (t == 0) {
+            extern __shared__ uint64_t sched_mem[];  // sched_small_bytes(G)
+            schedule_small(A.sa, reinterpret_cast<unsigned char *>(sched_mem));
+            return;
+        }
+        --t;
+    }
     if (t >= A.T) {
         if (deg || t - A.T >= n_extra)
             return;
@@ -734,7 +939,8 @@ static cudaError_t launch_fill(const FillArgs &A, cudaStream_t stream)
 {
     const int runs = A.T + (int)(A.N / ITEM_TICKETS) + 1;
     if (A.kr.anc)
-        launch_pdl(fill_tiles_kernel<true>, runs, TILE_THREADS, 0, stream, A);
+        launch_pdl(fill_tiles_kernel<true>, runs + (A.sched ? 1 : 0), TILE_THREADS,
+                   A.sched ? sched_small_bytes(A.sa.G) : 0, stream, A);
     else
         launch_pdl(fill_tiles_kernel<false>, runs, TILE_THREADS, 0, stream, A);
     return cudaGetLastError();
@@ -753,7 +959,7 @@ cudaError_t launch_draw_plain(const float *lw, int64_t N, DevSummary *sum, uint6
                          extra},
                 stream);
     const KeptRoute none{nullptr, nullptr, nullptr, 0, Balanced{0, 0}};
-    return launch_fill(FillArgs{lw, N, T, nd, sum, Ct, Tt, To, St, extra, out, none}, stream);
+    return launch_fill(FillArgs{lw, N, T, nd, sum, Ct, Tt, To, St, extra, out, none, 0, SchedArgs{}}, stream);
 }
 
 // ------------------------------------------------ two-stage RPA, stage 2
@@ -952,14 +1158,23 @@ __global__ void __launch_bounds__(TILE_THREADS, 3) group_fill_kernel(
     const float *__restrict__ lw, int64_t N, int32_t G, const int64_t *__restrict__ Tg,
     const uint64_t *__restrict__ Ct, const GroupGrid *__restrict__ grid, const int4 *__restrict__ split,
     int32_t n_workers, const DevSummary *__restrict__ sum, double ess_thr, int32_t *__restrict__ out,
-    int32_t *__restrict__ kept_anc, Balanced bl, int s)
+    int32_t *__restrict__ kept_anc, Balanced bl, int s, int sched, SchedArgs sa)
 {
     if (!pdl_wait())
         return;
     pdl_trigger();
+    int32_t block = blockIdx.x;
+    if (sched) {  // the first block runs the schedule
+        if (block == 0) {
+            extern __shared__ uint64_t sched_mem[];  // sched_small_bytes(G)
+            schedule_small(sa, reinterpret_cast<unsigned char *>(sched_mem));
+            return;
+        }
+        --block;
+    }
     __shared__ ParentSmem sm;
-    if ((int32_t)blockIdx.x >= n_workers) {  // a group block: one item, no loop
-        const GroupGrid gg = grid[blockIdx.x - n_workers];
+    if (block >= n_workers) {  // a group block: one item, no loop
+        const GroupGrid gg = grid[block - n_workers];
         const double ess = sum->ess;
         const int32_t deg = sum->degenerate;
         const float M = sum->M;
@@ -973,7 +1188,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 3) group_fill_kernel(
         return;
     const float M = sum->M;
     const int32_t n_items = sum->n_split + sum->n_runs;
-    for (int32_t it = (int32_t)blockIdx.x; it < n_items; it += n_workers) {
+    for (int32_t it = block; it < n_items; it += n_workers) {
         const int4 en = split[it];
         const GroupGrid gg = grid[en.y];
         if (en.x >= 0) {  // run en.z of a large group's part in tile en.x
@@ -998,22 +1213,6 @@ __global__ void __launch_bounds__(TILE_THREADS, 3) group_fill_kernel(
 // with the i-th receiver.  Output: new group offsets and the routing
 // segments (ticket start, slot start, length) with their copy work items
 // (GS and SGS: the links only, from schedule_links_balanced).
-struct SchedArgs {
-    int64_t N;
-    int32_t G;
-    int scheme;
-    const int64_t *goff;
-    int64_t *goff_new;
-    const int64_t *Tg;
-    uint64_t *key;      // [2 * G]  (sender keys, receiver keys)
-    int64_t *val;       // [5 * G]  (PS, PR, sent, recv, merge buffer)
-    int32_t *seg_chunk; // [2G + 2]
-    int64_t *seg_tick, *seg_dst, *seg_len;  // [2G + 1]
-    DevSummary *sum;
-    int links_only;  // the fill wrote the kept segments already: copy work items for the links only
-    Balanced bl;     // the balanced targets n_g
-};
-
 // block-wide exclusive scan of an int64 array in place (single block)
 __device__ void block_scan_i64(int64_t *a, int n, uint64_t *red, int64_t *total_out)
 {
@@ -1062,7 +1261,7 @@ __device__ void block_sort_u64(uint64_t *g, int n, uint64_t *sm, int cap)
             sm[i] = g[i];
     __syncthreads();
     const int t0 = threadIdx.x * SORT_PER;
-    {
+    if (t0 < n) {
         uint64_t k[SORT_PER];
         uint16_t id[SORT_PER];
 #pragma unroll
@@ -1153,20 +1352,6 @@ __device__ __forceinline__ int lower_bound_i64(const int64_t *a, int n, int64_t 
             lo = mid + 1;
         else
             hi = mid;
-    }
-    return lo;
-}
-
-// first index in sorted a[0..n) with a[i] > v (int32 values in shared memory)
-__device__ __forceinline__ int upper_bound_i32(const int32_t *a, int n, int32_t v)
-{
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (a[mid] > v)
-            hi = mid;
-        else
-            lo = mid + 1;
     }
     return lo;
 }
@@ -1592,6 +1777,9 @@ __global__ void __launch_bounds__(256) route_copy_kernel(const int32_t *__restri
                                                          const int64_t *__restrict__ seg_len, int64_t N,
                                                          DevSummary *__restrict__ sum)
 {
+    if (!pdl_wait())
+        return;
+    pdl_trigger();
     __shared__ int32_t sseg;
     const int32_t nb = sum->n_chunks;
     const int32_t nseg = seg_chunk[2 * G + 1];
@@ -2036,6 +2224,11 @@ __global__ void fill_f32_kernel(float *__restrict__ a, int64_t N, float v)
 cudaError_t resample_kernel_attributes()
 {
     cudaError_t e = cudaSuccess;
+    e = cudaFuncSetAttribute(fill_tiles_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sched_small_bytes(SCHED_SMALL));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(group_fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sched_small_bytes(SCHED_SMALL));
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(schedule_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)SORT_SMEM_BYTES);
@@ -2054,15 +2247,8 @@ static void launch_tile_tickets(ppf_ctx *c, double ess_thr, int rpa)
     c->launches += launch_scan(A, c->stream) - 1;
 }
 
-// The RPA schedule on the context's side stream, after the tile scan (an
-// event on the main stream), its completion recorded in ev_sched.
-static cudaError_t launch_schedule(ppf_ctx *c, int scheme, bool two_stage)
+static SchedArgs sched_args(ppf_ctx *c, int scheme, bool two_stage)
 {
-    cudaError_t e = cudaEventRecord(c->ev_scan, c->stream);
-    if (e == cudaSuccess)
-        e = cudaStreamWaitEvent(c->side_stream, c->ev_scan, 0);
-    if (e != cudaSuccess)
-        return e;
     SchedArgs A;
     A.N = c->N;
     A.G = c->G;
@@ -2079,8 +2265,20 @@ static cudaError_t launch_schedule(ppf_ctx *c, int scheme, bool two_stage)
     A.sum = c->sum;
     A.links_only = A.scheme != PPF_RPA_LGS;
     A.bl = balanced_layout(c->N, c->G);
-    const size_t sched_smem = sched_smem_bytes(c->G);
-    schedule_kernel<<<1, 1024, sched_smem, c->side_stream>>>(A);
+    return A;
+}
+
+// The RPA schedule of more than SCHED_SMALL groups, or of LGS, on the context's
+// side stream, after the tile scan (an event on the main stream), its
+// completion recorded in ev_sched.
+static cudaError_t launch_schedule(ppf_ctx *c, const SchedArgs &A)
+{
+    cudaError_t e = cudaEventRecord(c->ev_scan, c->stream);
+    if (e == cudaSuccess)
+        e = cudaStreamWaitEvent(c->side_stream, c->ev_scan, 0);
+    if (e != cudaSuccess)
+        return e;
+    schedule_kernel<<<1, 1024, sched_smem_bytes(c->G), c->side_stream>>>(A);
     e = cudaGetLastError();
     if (e == cudaSuccess)
         e = cudaEventRecord(c->ev_sched, c->side_stream);
@@ -2093,7 +2291,7 @@ cudaError_t launch_resample_global(ppf_ctx *c, int scheme, double ess_thr)
     const float *lw = c->state[c->cur] + 5 * c->N;
     const int T = c->T;
     prof_mark(c, PH_RESAMPLE, 0);
-    c->launches += rpa ? 5 : 3;
+    c->launches += rpa ? 4 : 3;
     if (rpa)
         launch_pdl(tile_group_totals_kernel, T, TILE_THREADS, 0, c->stream, lw, c->N, (const DevSummary *)c->sum,
                    ess_thr, c->sc.Qt, c->sc.St, (const int64_t *)c->goff, c->G, c->sc.Cbl, c->sc.tile_g);
@@ -2103,16 +2301,19 @@ cudaError_t launch_resample_global(ppf_ctx *c, int scheme, double ess_thr)
     launch_tile_tickets(c, ess_thr, rpa ? 1 : 0);
     int32_t *out = rpa ? c->anc_sys : c->anc;
     const bool two_stage = (scheme >= PPF_RPA2_GS && scheme <= PPF_RPA2_LGS);
-    if (rpa) {
-        // The routing schedule needs only the tile scan (offspring counts per
-        // group), not the fill: it runs on a side stream, one block on one
-        // SM, while the fill runs on the others; the copy joins them.
-        cudaError_t e0 = launch_schedule(c, scheme, two_stage);
-        if (e0 != cudaSuccess)
-            return e0;
-    }
     // GS and SGS: the kept tickets go straight to their balanced slots
     const bool kept_direct = rpa && scheme != PPF_RPA_LGS && scheme != PPF_RPA2_LGS;
+    // The routing schedule needs only the tile scan (offspring counts per
+    // group), not the fill, and runs beside it on one SM: as the fill's first
+    // block where its lists are small, else on a side stream that the copy joins.
+    const bool in_fill = kept_direct && c->G <= SCHED_SMALL;
+    const SchedArgs sa = rpa ? sched_args(c, scheme, two_stage) : SchedArgs{};
+    if (rpa && !in_fill) {
+        cudaError_t e0 = launch_schedule(c, sa);
+        if (e0 != cudaSuccess)
+            return e0;
+        c->launches += 1;
+    }
     if (two_stage) {  // stage 2: every group draws its own offspring
         int4 *split = reinterpret_cast<int4 *>(c->sc.split);
         group_grid_kernel<<<(c->G + 255) / 256, 256, 0, c->stream>>>(
@@ -2121,15 +2322,16 @@ cudaError_t launch_resample_global(ppf_ctx *c, int scheme, double ess_thr)
         launch_pdl(split_runs_kernel, c->num_sms, 256, 0, c->stream, (const uint64_t *)c->sc.Ct,
                    (const GroupGrid *)c->sc.ggrid, split, c->sum, ess_thr);
         const int n_workers = 4 * c->num_sms;
-        launch_pdl(group_fill_kernel, n_workers + c->G, TILE_THREADS, 0, c->stream, lw, c->N, c->G,
+        launch_pdl(group_fill_kernel, n_workers + c->G + (in_fill ? 1 : 0), TILE_THREADS,
+                   in_fill ? sched_small_bytes(c->G) : 0, c->stream, lw, c->N, c->G,
                    (const int64_t *)c->sc.Tg, (const uint64_t *)c->sc.Ct, (const GroupGrid *)c->sc.ggrid,
                    (const int4 *)split, n_workers, (const DevSummary *)c->sum, ess_thr, out,
-                   kept_direct ? c->anc : nullptr, balanced_layout(c->N, c->G), scale_bits(c->N));
+                   kept_direct ? c->anc : nullptr, balanced_layout(c->N, c->G), scale_bits(c->N), in_fill ? 1 : 0, sa);
         c->launches += 2;
     } else {
         const KeptRoute kr{kept_direct ? c->anc : nullptr, c->sc.Tg, c->sc.tile_g, c->G, balanced_layout(c->N, c->G)};
         const FillArgs A{lw, c->N, T, make_divisor((uint32_t)c->N), c->sum, c->sc.Ct, c->sc.Tt, c->sc.To, c->sc.St,
-                         reinterpret_cast<const int2 *>(c->sc.extra), out, kr};
+                         reinterpret_cast<const int2 *>(c->sc.extra), out, kr, in_fill ? 1 : 0, sa};
         launch_fill(A, c->stream);
     }
     cudaError_t e = cudaGetLastError();
@@ -2137,14 +2339,20 @@ cudaError_t launch_resample_global(ppf_ctx *c, int scheme, double ess_thr)
         prof_mark(c, PH_RESAMPLE, 1);
         return e;
     }
-    e = cudaStreamWaitEvent(c->stream, c->ev_sched, 0);  // join the schedule
-    if (e != cudaSuccess)
-        return e;
+    if (!in_fill) {
+        e = cudaStreamWaitEvent(c->stream, c->ev_sched, 0);  // join the schedule
+        if (e != cudaSuccess)
+            return e;
+    }
     const int max_chunks = 2 * c->G + 1 + (int)((c->N + COPY_CHUNK - 1) / COPY_CHUNK);
     const int gcopy = max_chunks < 8 * c->num_sms ? max_chunks : 8 * c->num_sms;
-    route_copy_kernel<<<gcopy, 256, 0, c->stream>>>(c->anc_sys, c->anc, c->G, c->sc.seg_chunk,
-                                                         c->sc.seg_tick, c->sc.seg_dst, c->sc.seg_len, c->N,
-                                                         c->sum);
+    if (in_fill)
+        launch_pdl(route_copy_kernel, gcopy, 256, 0, c->stream, (const int32_t *)c->anc_sys, c->anc, c->G,
+                   (const int32_t *)c->sc.seg_chunk, (const int64_t *)c->sc.seg_tick, (const int64_t *)c->sc.seg_dst,
+                   (const int64_t *)c->sc.seg_len, c->N, c->sum);
+    else
+        route_copy_kernel<<<gcopy, 256, 0, c->stream>>>(c->anc_sys, c->anc, c->G, c->sc.seg_chunk, c->sc.seg_tick,
+                                                         c->sc.seg_dst, c->sc.seg_len, c->N, c->sum);
     prof_mark(c, PH_RESAMPLE, 1);
     return cudaGetLastError();
 }

@@ -66,3 +66,23 @@ def test_rna_block_sizes(orc, group):
     pf = ppf.ParticleFilter(gm, 3 * group + 7, group_size=group)
     lockstep(pf, gm, om, mv.frames, torch.from_numpy(mv.frames).cuda(), orc.RNA, K=2, alpha=0.25)
     pf.close()
+
+
+@pytest.mark.parametrize("scheme", ["rpa_gs", "rpa_sgs", "rpa2_sgs"])
+@pytest.mark.parametrize("groups", [1, 2, 33, 64, 65, 2048, 2049])
+def test_schedule_group_counts(orc, groups, scheme):
+    """The GS and SGS schedule in the fill's first block (up to 2048 groups)
+    and on the side stream (above): counts at the edges of the sort's powers of
+    two and of the rule, groups of 5 particles and one ragged."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import synth
+    import paper_1310_5045_gb300 as ppf
+    from gpu_common import lockstep, paired_models
+    mv = synth.make_movie(W=64, H=64, K=2, seed=4)
+    gm, om = paired_models(ppf, seed=groups, width=64, height=64, patch_radius=2)
+    pf = ppf.ParticleFilter(gm, 5 * groups - (1 if groups > 1 else 0), group_size=5)
+    assert len(pf.groups()) - 1 == groups
+    lockstep(pf, gm, om, mv.frames, torch.from_numpy(mv.frames).cuda(), getattr(orc, scheme.upper()), K=2)
+    pf.close()
