@@ -188,9 +188,9 @@ ppf_status ppf_create(const ppf_model *m, int64_t n, int32_t group_size, void *s
     c->pad = 2 * m->patch_radius;
     // row pitch (in pixel pairs): the padded width plus one zero column (the
     // frame is held as pairs (Z(col), Z(col + 1)), so that the patch sum reads
-    // aligned pixel pairs), rounded up to even so that a row is a multiple of
-    // 16 bytes (the tensor copies of the binned path need it)
-    c->Wp = (m->width + 2 * c->pad + 2) & ~1;
+    // aligned pixel pairs), spread over the banks; even, so that a row is a
+    // multiple of 16 bytes (the tensor copies of the binned path need it)
+    c->Wp = spread_pitch((m->width + 2 * c->pad + 2) & ~1, 2);
     c->Hp = m->height + 2 * c->pad;
     c->frame_bytes = (size_t)m->width * m->height * dtype_size(m->frame_dtype);
     c->mode = MODE_CARRY;

@@ -100,6 +100,7 @@ struct ppf_batch {
     int4 *fsc;                         // device [F]: the ticket counts' scale (TicketScale)
     uint64_t *fQu;                     // device [4F]: per filter Q_f, u_f, Q_f / n_f, Q_f mod n_f
     ppf::Partial *upart;               // device [U]
+    int32_t *next_unit;                // device: the next work unit no warp has taken
     ppf::FilterSummary *fsum;          // device [F]
     ppf::FilterSummary *fsum_host;     // pinned [F]
     ppf::FilterSummary *fsum_run;      // device [K x F] of the last graph run
@@ -179,8 +180,11 @@ __global__ void batch_advance(BatchCursor *c)
 
 template <typename T>
 __global__ void batch_prepare_kernel(const BatchCursor *__restrict__ cur, float *__restrict__ Zp, int32_t F, int W,
-                                     int H, int Wp, int Hp, int pad, const FilterParams *__restrict__ fp)
+                                     int H, int Wp, int Hp, int pad, const FilterParams *__restrict__ fp,
+                                     int32_t *__restrict__ next_unit)
 {
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        *next_unit = 0;  // the step after this takes the units from the first
     // one warp per padded row (F * Hp rows), lanes across its columns; each
     // element is the pixel pair (Z(col), Z(col + 1)) minus the background
     const T *Z = reinterpret_cast<const T *>(cur->frames + cur->frame_bytes * cur->t);
@@ -217,13 +221,17 @@ struct BatchStepArgs {
     const float *__restrict__ Zp;
     Partial *__restrict__ part;
     int32_t *flags;             // FLAG_INTERNAL from a failed debug check
+    int32_t *next_unit;
 };
 
 // Persistent SIS step over all work units of all filters.  A unit is a run
 // of at most `unit` particles of one filter and belongs to one warp: the warp
 // steps its particles (the next slot's ancestor loaded one iteration ahead)
 // and reduces their weight statistics with shuffles into the unit's partial,
-// with no block-wide synchronisation.
+// with no block-wide synchronisation.  Warps take units from a counter, the
+// next one while they step the current: units differ in size, and the blocks
+// that do not fit the SMs at once would leave a second, nearly empty wave of
+// a fixed share each (1024 filters, 12M particles: 343 us a frame then).
 template <int R>
 __global__ void batch_step_kernel(BatchStepArgs a)
 {
@@ -237,8 +245,13 @@ __global__ void batch_step_kernel(BatchStepArgs a)
     const float *__restrict__ slw = src + 5 * (size_t)N;
     __shared__ float kcs[32][MAX_RADIUS];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int32_t nwarps = (int32_t)(gridDim.x * (blockDim.x >> 5));
-    for (int32_t u = (int32_t)(blockIdx.x * (blockDim.x >> 5)) + wib; u < a.U; u += nwarps) {
+    auto take = [&]() { return lane == 0 ? atomicAdd(a.next_unit, 1) : 0; };
+    int32_t taken = take();
+    for (;;) {
+        const int32_t u = __shfl_sync(0xffffffffu, taken, 0);
+        if (u >= a.U)
+            break;
+        taken = take();
         const int32_t f = a.unit_f[u];
         const FilterParams *__restrict__ P = a.fp + f;
         const uint32_t off = (uint32_t)P->off, nf = (uint32_t)P->n;
@@ -270,12 +283,12 @@ __global__ void batch_step_kernel(BatchStepArgs a)
             const float vx = __ldg(svx + p), vy = __ldg(svy + p);
             const float I0 = __ldg(sI + p);
             const float lwp = carry ? __ldg(slw + p) : 0.0f;
-            uint32_t fl[6];
-            prop_fields(draw(seed, i - off, frame, fid, PURPOSE_PROP, 0), fl);
+            float fl[6];
+            prop_uniforms(draw(seed, i - off, frame, fid, PURPOSE_PROP, 0), fl);
             float e0, e1, e2, e3, e4, e5;
-            box_muller(u21(fl[0]), u21(fl[1]), e0, e1);
-            box_muller(u21(fl[2]), u21(fl[3]), e2, e3);
-            box_muller(u21(fl[4]), u21(fl[5]), e4, e5);
+            box_muller(fl[0], fl[1], e0, e1);
+            box_muller(fl[2], fl[3], e2, e3);
+            box_muller(fl[4], fl[5], e4, e5);
             float v[5];
             v[0] = fmaf(sm, e0, x + vx);
             v[1] = fmaf(sm, e1, y + vy);
@@ -615,6 +628,7 @@ cudaError_t launch_batch_step(ppf_batch *b, bool commit)
     a.fkeep = b->fkeep;
     a.Zp = b->Zp;
     a.flags = b->flags;
+    a.next_unit = b->next_unit;
     a.part = b->upart;
     int grid = b->num_sms * b->bps;
     if (grid > b->U)
@@ -646,15 +660,15 @@ cudaError_t launch_batch_prepare(ppf_batch *b)
     switch (b->dtype) {
     case PPF_BF16:
         batch_prepare_kernel<__nv_bfloat16><<<grid, 256, 0, b->stream>>>(b->cursor, b->Zp, b->F, b->W, b->H, b->Wp,
-                                                                         b->Hp, b->pad, b->fp);
+                                                                         b->Hp, b->pad, b->fp, b->next_unit);
         break;
     case PPF_F16:
         batch_prepare_kernel<__half><<<grid, 256, 0, b->stream>>>(b->cursor, b->Zp, b->F, b->W, b->H, b->Wp, b->Hp,
-                                                                  b->pad, b->fp);
+                                                                  b->pad, b->fp, b->next_unit);
         break;
     default:
         batch_prepare_kernel<float><<<grid, 256, 0, b->stream>>>(b->cursor, b->Zp, b->F, b->W, b->H, b->Wp, b->Hp,
-                                                                 b->pad, b->fp);
+                                                                 b->pad, b->fp, b->next_unit);
     }
     b->launches += 1;
     return cudaGetLastError();
@@ -711,7 +725,7 @@ void free_batch(ppf_batch *b)
     if (b->gstream)
         cudaStreamDestroy(b->gstream);
     void *p[] = {b->fp, b->state[0], b->state[1], b->anc, b->Zp, b->unit_f, b->unit_lo, b->unit_n, b->fu_off,
-                 b->upart, b->fsum, b->flags, b->fkeep, b->fsum_run, b->cursor, b->tile_f, b->tile_lo, b->tile_n,
+                 b->upart, b->next_unit, b->fsum, b->flags, b->fkeep, b->fsum_run, b->cursor, b->tile_f, b->tile_lo, b->tile_n,
                  b->ft_off,
                  b->tQ, b->tC, b->tT, b->tO, b->tS, b->fsc, b->fQu};
     for (void *q : p)
@@ -768,7 +782,8 @@ ppf_status ppf_batch_create(const ppf_model *models, const int64_t *n, int32_t F
     b->H = m0.height;
     b->r = m0.patch_radius;
     b->pad = 2 * b->r;
-    b->Wp = b->W + 2 * b->pad + 1;  // pixel pairs per row: one zero column past the padded frame
+    // pixel pairs per row: one zero column past the padded frame, spread over the banks
+    b->Wp = spread_pitch(b->W + 2 * b->pad + 1, 1);
     b->Hp = b->H + 2 * b->pad;
     b->dtype = m0.frame_dtype;
     b->frame_bytes = (size_t)b->W * b->H * (b->dtype == PPF_F32 ? 4 : 2);
@@ -819,7 +834,7 @@ ppf_status ppf_batch_create(const ppf_model *models, const int64_t *n, int32_t F
         dmalloc(&b->state[1], 6 * Ntot) != cudaSuccess || dmalloc(&b->anc, Ntot) != cudaSuccess ||
         dmalloc(&b->Zp, 2 * (size_t)F * b->Wp * b->Hp) != cudaSuccess || dmalloc(&b->fu_off, F + 1) != cudaSuccess ||
         dmalloc(&b->fsum, F) != cudaSuccess || dmalloc(&b->flags, 1) != cudaSuccess ||
-        dmalloc(&b->fkeep, F) != cudaSuccess ||
+        dmalloc(&b->fkeep, F) != cudaSuccess || dmalloc(&b->next_unit, 1) != cudaSuccess ||
         dmalloc(&b->cursor, 1) != cudaSuccess ||
         cudaMallocHost((void **)&b->fsum_host, sizeof(FilterSummary) * F) != cudaSuccess ||
         dmalloc(&dv0A, 2 * (size_t)F) != cudaSuccess)
@@ -1007,13 +1022,17 @@ ppf_status ppf_batch_autotune(ppf_batch *b, const void *frames_dev, int32_t k, i
             e = build_units(b, un);
         b->block = bl;
         b->bps = bp;
+        auto step = [&]() {  // from the first unit, as after a frame's preparation
+            const cudaError_t r = cudaMemsetAsync(b->next_unit, 0, sizeof(int32_t), b->stream);
+            return r == cudaSuccess ? launch_batch_step(b, false) : r;
+        };
         if (e == cudaSuccess)
-            e = launch_batch_step(b, false);
+            e = step();
         float best_ms = 1e30f;
         for (int trial = 0; trial < 3 && e == cudaSuccess; ++trial) {
             e = cudaEventRecord(e0, b->stream);
             for (int rep = 0; rep < 3 && e == cudaSuccess; ++rep)
-                e = launch_batch_step(b, false);
+                e = step();
             if (e == cudaSuccess)
                 e = cudaEventRecord(e1, b->stream);
             if (e == cudaSuccess)

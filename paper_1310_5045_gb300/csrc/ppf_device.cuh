@@ -125,25 +125,25 @@ __device__ __forceinline__ float u01(uint32_t r)
     return __uint2float_rn(2u * (r >> 9) + 1u) * 0x1p-24f;
 }
 
-// odd multiple of 2^-22 in (0, 1) from a 21-bit field; exact in float32
-__device__ __forceinline__ float u21(uint32_t f)
+// The six uniforms of one Philox block (word 0 least significant): field k
+// holds bits [21k, 21k + 21) of the 128-bit block and gives the odd multiple
+// (2 f + 1) 2^-22 of 2^-22 in (0, 1).  The field is shifted to the top 21 of
+// the 23 mantissa bits of 1 + (2 f + 1) 2^-22 and 1 subtracted, both exact: a
+// shift, a mask-or and an addition instead of an integer conversion, which
+// runs on the quarter-rate pipe.
+__device__ __forceinline__ float field_uniform(uint32_t w)  // field at bits 2..22
 {
-    return __uint2float_rn(2u * f + 1u) * 0x1p-22f;
+    return __fsub_rn(__uint_as_float((w & 0x7FFFFCu) | 0x3F800002u), 1.0f);
 }
 
-// The six 21-bit fields of one Philox block (word 0 least significant):
-// field k holds bits [21k, 21k + 21) of the 128-bit block.
-__device__ __forceinline__ void prop_fields(uint4 r, uint32_t f[6])
+__device__ __forceinline__ void prop_uniforms(uint4 r, float u[6])
 {
-    const uint64_t lo = (uint64_t)r.x | ((uint64_t)r.y << 32);
-    const uint64_t hi = (uint64_t)r.z | ((uint64_t)r.w << 32);
-    const uint64_t m = 0x1FFFFFull;
-    f[0] = (uint32_t)(lo & m);
-    f[1] = (uint32_t)((lo >> 21) & m);
-    f[2] = (uint32_t)((lo >> 42) & m);
-    f[3] = (uint32_t)(((lo >> 63) | (hi << 1)) & m);
-    f[4] = (uint32_t)((hi >> 20) & m);
-    f[5] = (uint32_t)((hi >> 41) & m);
+    u[0] = field_uniform(r.x << 2);
+    u[1] = field_uniform(__funnelshift_r(r.x, r.y, 19));
+    u[2] = field_uniform(r.y >> 8);
+    u[3] = field_uniform(__funnelshift_r(r.y, r.z, 29));
+    u[4] = field_uniform(__funnelshift_r(r.z, r.w, 18));
+    u[5] = field_uniform(r.w >> 7);
 }
 
 // Box-Muller: rho = sqrt(-2 ln u1) (accurate log: u1 -> 1 needs it), angle

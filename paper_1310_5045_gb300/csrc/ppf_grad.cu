@@ -290,11 +290,11 @@ __global__ void __launch_bounds__(256, R <= 5 ? 2 : 1) grad_step_kernel(GradArgs
         const float x = __ldg(a.src + p), y = __ldg(a.src + N + p);
         const float vx = __ldg(a.src + 2 * N + p), vy = __ldg(a.src + 3 * N + p);
         const float tx = a.first ? 0.0f : __ldg(a.tsrc + p), ty = a.first ? 0.0f : __ldg(a.tsrc + N + p);
-        uint32_t f[6];
-        prop_fields(philox_rk(make_uint4((uint32_t)i, a.frame, a.fid, PURPOSE_PROP << 8), a.rk), f);
+        float f[6];
+        prop_uniforms(philox_rk(make_uint4((uint32_t)i, a.frame, a.fid, PURPOSE_PROP << 8), a.rk), f);
         float e0, e1, e2, e3;
-        box_muller(u21(f[0]), u21(f[1]), e0, e1);
-        box_muller(u21(f[2]), u21(f[3]), e2, e3);
+        box_muller(f[0], f[1], e0, e1);
+        box_muller(f[2], f[3], e2, e3);
         const float nx = fmaf(a.sm, e0, x + vx), ny = fmaf(a.sm, e1, y + vy);
         const float ntx = tx + e0, nty = ty + e1;
         float d[6];

@@ -19,6 +19,21 @@ struct NvtxRange {
     NvtxRange &operator=(const NvtxRange &) = delete;
 };
 
+// The smallest pitch from `pairs` on, in steps of `step`, that spreads the rows
+// of a patch over the L1's 16 eight-byte banks.  A warp's lanes read the same
+// patch row from anchors a few pixels apart in x and y: with a pitch of 0 (mod
+// 16) all their rows meet in the same banks, at 8 every other one, near 0 rows
+// next to each other overlap.  Direct step of 4M particles at r = 5 by the
+// pitch mod 16: 0 166 us, 8 122, 2 and 14 118, 4, 6, 10 and 12 114; at r = 7:
+// 0 278, 8 188, 2 and 14 173, the others 150 to 153; the batched frame of 1024
+// filters: 0 5018, 1, 8 and 15 4290, the others 3800 to 3900.
+inline int spread_pitch(int pairs, int step)
+{
+    while (pairs % 16 <= 2 || pairs % 16 == 8 || pairs % 16 >= 14)
+        pairs += step;
+    return pairs;
+}
+
 constexpr int TILE = 4096;          // particles per resampling tile (256 threads x 16)
 constexpr int TILE_THREADS = 256;
 constexpr int TILE_ITEMS = TILE / TILE_THREADS;

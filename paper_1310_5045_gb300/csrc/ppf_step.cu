@@ -124,12 +124,12 @@ __device__ __forceinline__ Propagated propagate_slot(const StepArgs &a, int mode
         r.lwp = 0.0f;
     else
         r.lwp = __ldg(a.lwp + i);
-    uint32_t f[6];
-    prop_fields(philox_rk(make_uint4(i, a.frame, a.fid, PURPOSE_PROP << 8), a.rk), f);
+    float f[6];
+    prop_uniforms(philox_rk(make_uint4(i, a.frame, a.fid, PURPOSE_PROP << 8), a.rk), f);
     float e0, e1, e2, e3, e4, e5;
-    box_muller(u21(f[0]), u21(f[1]), e0, e1);
-    box_muller(u21(f[2]), u21(f[3]), e2, e3);
-    box_muller(u21(f[4]), u21(f[5]), e4, e5);
+    box_muller(f[0], f[1], e0, e1);
+    box_muller(f[2], f[3], e2, e3);
+    box_muller(f[4], f[5], e4, e5);
     r.v[0] = fmaf(a.sm, e0, x + vx);
     r.v[1] = fmaf(a.sm, e1, y + vy);
     r.v[2] = fmaf(a.sv, e2, vx);
@@ -290,12 +290,12 @@ __global__ void __launch_bounds__(256, 3) step_kernel(StepArgs a, int phase)
                 lwp = 0.0f;
             else
                 lwp = __ldg(a.lwp + i);
-            uint32_t f[6];
-            prop_fields(philox_rk(make_uint4((uint32_t)i, a.frame, a.fid, PURPOSE_PROP << 8), a.rk), f);
+            float f[6];
+            prop_uniforms(philox_rk(make_uint4((uint32_t)i, a.frame, a.fid, PURPOSE_PROP << 8), a.rk), f);
             float e0, e1, e2, e3, e4, e5;
-            box_muller(u21(f[0]), u21(f[1]), e0, e1);
-            box_muller(u21(f[2]), u21(f[3]), e2, e3);
-            box_muller(u21(f[4]), u21(f[5]), e4, e5);
+            box_muller(f[0], f[1], e0, e1);
+            box_muller(f[2], f[3], e2, e3);
+            box_muller(f[4], f[5], e4, e5);
             float v[5];
             v[0] = fmaf(a.sm, e0, x + vx);
             v[1] = fmaf(a.sm, e1, y + vy);
