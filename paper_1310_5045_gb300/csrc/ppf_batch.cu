@@ -228,10 +228,11 @@ struct BatchStepArgs {
 // of at most `unit` particles of one filter and belongs to one warp: the warp
 // steps its particles (the next slot's ancestor loaded one iteration ahead)
 // and reduces their weight statistics with shuffles into the unit's partial,
-// with no block-wide synchronisation.  Warps take units from a counter, the
-// next one while they step the current: units differ in size, and the blocks
-// that do not fit the SMs at once would leave a second, nearly empty wave of
-// a fixed share each (1024 filters, 12M particles: 343 us a frame then).
+// with no block-wide synchronisation.  The grid is what fits the SMs at once
+// (a second wave of blocks would be nearly empty); every warp begins with one
+// unit, dealt so that few units spread over the SMs, and takes the others from
+// a counter, since units differ in size (1024 filters, 12M
+// particles: 343 us a frame with a fixed share per warp of four blocks per SM).
 template <int R>
 __global__ void batch_step_kernel(BatchStepArgs a)
 {
@@ -245,13 +246,13 @@ __global__ void batch_step_kernel(BatchStepArgs a)
     const float *__restrict__ slw = src + 5 * (size_t)N;
     __shared__ float kcs[32][MAX_RADIUS];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    auto take = [&]() { return lane == 0 ? atomicAdd(a.next_unit, 1) : 0; };
-    int32_t taken = take();
-    for (;;) {
-        const int32_t u = __shfl_sync(0xffffffffu, taken, 0);
-        if (u >= a.U)
-            break;
-        taken = take();
+    // the first unit: a block's warps begin with consecutive units (mostly of
+    // one filter, so of one frame), at most `deal` of them
+    const int32_t per_block = (a.U + (int32_t)gridDim.x - 1) / (int32_t)gridDim.x;
+    const int32_t deal = per_block < (int32_t)(blockDim.x >> 5) ? per_block : (int32_t)(blockDim.x >> 5);
+    const int32_t dealt = deal * (int32_t)gridDim.x;
+    int32_t u = wib < deal ? (int32_t)blockIdx.x * deal + wib : a.U;
+    while (u < a.U) {
         const int32_t f = a.unit_f[u];
         const FilterParams *__restrict__ P = a.fp + f;
         const uint32_t off = (uint32_t)P->off, nf = (uint32_t)P->n;
@@ -306,6 +307,10 @@ __global__ void batch_step_kernel(BatchStepArgs a)
             else
                 acc.add_prev_zero();
         }
+        // the next unit (not earlier: a unit taken ahead would wait for this one)
+        const int32_t next = lane == 0 ? dealt + atomicAdd(a.next_unit, 1) : 0;
+        const int32_t mine = u;
+        u = __shfl_sync(0xffffffffu, next, 0);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1)
             acc.shfl_merge(o);
@@ -318,7 +323,7 @@ __global__ void batch_step_kernel(BatchStepArgs a)
                 q.s[c] = acc.s[c];
             q.mp = acc.mp;
             q.sp = acc.sp;
-            a.part[u] = q;
+            a.part[mine] = q;
         }
     }
 }
@@ -602,8 +607,12 @@ cudaError_t build_tiles(ppf_batch *b)
 }
 
 template <int R>
-void launch_batch_step_r(const BatchStepArgs &a, int grid, int block, cudaStream_t s)
+void launch_batch_step_r(const BatchStepArgs &a, int num_sms, int bps, int block, cudaStream_t s)
 {
+    int fit = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, batch_step_kernel<R>, block, 0);
+    fit = fit < 1 ? 1 : (fit < bps ? fit : bps);
+    const int grid = num_sms * fit < a.U ? num_sms * fit : a.U;
     batch_step_kernel<R><<<grid, block, 0, s>>>(a);
 }
 
@@ -630,19 +639,16 @@ cudaError_t launch_batch_step(ppf_batch *b, bool commit)
     a.flags = b->flags;
     a.next_unit = b->next_unit;
     a.part = b->upart;
-    int grid = b->num_sms * b->bps;
-    if (grid > b->U)
-        grid = b->U;
     switch (b->r) {
-    case 0: launch_batch_step_r<0>(a, grid, b->block, b->stream); break;
-    case 1: launch_batch_step_r<1>(a, grid, b->block, b->stream); break;
-    case 2: launch_batch_step_r<2>(a, grid, b->block, b->stream); break;
-    case 3: launch_batch_step_r<3>(a, grid, b->block, b->stream); break;
-    case 4: launch_batch_step_r<4>(a, grid, b->block, b->stream); break;
-    case 5: launch_batch_step_r<5>(a, grid, b->block, b->stream); break;
-    case 6: launch_batch_step_r<6>(a, grid, b->block, b->stream); break;
-    case 7: launch_batch_step_r<7>(a, grid, b->block, b->stream); break;
-    default: launch_batch_step_r<8>(a, grid, b->block, b->stream); break;
+    case 0: launch_batch_step_r<0>(a, b->num_sms, b->bps, b->block, b->stream); break;
+    case 1: launch_batch_step_r<1>(a, b->num_sms, b->bps, b->block, b->stream); break;
+    case 2: launch_batch_step_r<2>(a, b->num_sms, b->bps, b->block, b->stream); break;
+    case 3: launch_batch_step_r<3>(a, b->num_sms, b->bps, b->block, b->stream); break;
+    case 4: launch_batch_step_r<4>(a, b->num_sms, b->bps, b->block, b->stream); break;
+    case 5: launch_batch_step_r<5>(a, b->num_sms, b->bps, b->block, b->stream); break;
+    case 6: launch_batch_step_r<6>(a, b->num_sms, b->bps, b->block, b->stream); break;
+    case 7: launch_batch_step_r<7>(a, b->num_sms, b->bps, b->block, b->stream); break;
+    default: launch_batch_step_r<8>(a, b->num_sms, b->bps, b->block, b->stream); break;
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || !commit)
