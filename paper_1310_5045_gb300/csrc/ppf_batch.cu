@@ -296,7 +296,11 @@ __global__ void batch_step_kernel(BatchStepArgs a)
             v[2] = fmaf(sv, e2, vx);
             v[3] = fmaf(sv, e3, vy);
             v[4] = fmaf(sIn, e4, I0);
-            const float lw = lwp + patch_loglik<R, false>(geom, v[0], v[1], v[4]);
+            // Packed FMAs where their operand pairs fit the register limit: 8
+            // frames of 1500 filters at radius 4 take 4521 us (scalar 4612), 4
+            // frames of 448 at radius 3 886 us (902); radius 5 would need 84
+            // registers, a resident block less.
+            const float lw = lwp + patch_loglik<R, (R <= 4)>(geom, v[0], v[1], v[4]);
 #pragma unroll
             for (int c = 0; c < 5; ++c)
                 dst[(size_t)c * N + i] = v[c];

@@ -179,9 +179,9 @@ __device__ __forceinline__ bool patch_setup(const PatchGeom &a, float x, float y
 // r_j = (sum_k gx_2k Zb(2k, j) + gx_P-1 Zb(P-1, j), sum_k gx_2k+1 Zb(2k+1, j)),
 // k over the P / 2 full column pairs; then b = sum_j gy_j r_j lane by lane and
 // B = b.x + b.y.  PACKED computes the two lanes with packed two-lane FMAs
-// over the pixel pairs; the scalar form (kept by the batched step, whose
-// warp-per-unit kernel ran slower with packed FMAs) performs the same
-// roundings in the same order, so both give the same bits.
+// over the pixel pairs; the scalar form (kept by the batched step at radii
+// above 4, where the packed operands cost it a resident block) performs the
+// same roundings in the same order, so both give the same bits.
 //
 // patch_rows takes the first pair of the window's first row and the row pitch
 // (in pairs); SMEM reads a window staged in shared memory with plain loads,
