@@ -62,7 +62,7 @@ void free_all(ppf_ctx *c)
                     c->state[0], c->state[1], c->anc, c->anc_sys, c->lwp, c->goff, c->goff_new, c->ring, c->succ, c->Zp,
                     c->frame_buf[0], c->frame_buf[1], c->lmap, c->part, c->sum, c->est_dev, c->sc.Qt, c->sc.St, c->sc.Ct, c->sc.Tt, c->sc.To, c->sc.extra, c->sc.Cbl,
                     c->sc.Tg, c->sc.tile_g, c->sc.ggrid, c->sc.split, c->sc.skey, c->sc.sval, c->sc.seg_tick, c->sc.seg_dst, c->sc.seg_len,
-                    c->sc.seg_chunk, c->bin_key, c->bin_l, c->bin_tot, c->bin_item, c->bin_rec};
+                    c->sc.seg_chunk, c->bin_key, c->bin_l, c->bin_tot, c->bin_rec};
     for (void *p : ptrs)
         if (p)
             cudaFree(p);
@@ -488,19 +488,14 @@ ppf_status ppf_set_particles(ppf_ctx *c, const float *state_dev, const int32_t *
                        c->stream));
     if (anc_dev)
         CK(cudaMemcpyAsync(c->anc, anc_dev, sizeof(int32_t) * c->N, cudaMemcpyDeviceToDevice, c->stream));
-    else
-        CK(ppf::launch_identity(c, c->anc));
     if (lwp_dev) {
         CK(cudaMemcpyAsync(c->lwp, lwp_dev, sizeof(float) * c->N, cudaMemcpyDeviceToDevice, c->stream));
         c->mode = MODE_EXPLICIT;
     } else {
         c->mode = anc_dev ? MODE_UNIFORM : MODE_CARRY;
     }
-    const int32_t zero = 0;
-    CK(cudaMemcpyAsync((char *)c->sum + offsetof(DevSummary, degenerate), &zero, sizeof(zero),
-                       cudaMemcpyHostToDevice, c->stream));
     // particles of unknown spread: the next step bins them (and measures)
-    CK(ppf::bin_set_next(c, 1));
+    CK(ppf::launch_restart(c, !anc_dev));
     c->weighted = false;
     return PPF_OK;
 }

@@ -10,12 +10,11 @@
 //      turns the bin sizes into bin starts, takes chunks of slots, ranks them
 //      by bin in shared memory and reserves one range per bin with one
 //      atomic, so a bin's records from one chunk are written contiguously;
-//      the slot keeps its record's place; the last block cuts the bins into
-//      work items;
+//      the slot keeps its record's place;
 //   3. runs the likelihood over work items of one bin: the tile's window
-//      (the tile plus the patch halo) is copied into shared memory by the
-//      tensor-memory accelerator (cp.async.bulk.tensor, completion on an
-//      mbarrier), the next item's window copied while this one is summed,
+//      (the tile plus the patch halo) and the item's records are copied into
+//      shared memory by the tensor-memory accelerator (cp.async.bulk,
+//      completion on an mbarrier), the next item's while this one is summed,
 //      every patch read comes from shared memory, and l is written in bin
 //      order;
 //   4. sums in the direct path's slot order (the step kernel's phase 1),
@@ -36,7 +35,7 @@
 
 namespace ppf {
 
-constexpr int BIN_ITEM = 4096;        // records per likelihood work item
+constexpr int BIN_ITEM = 1280;        // records per likelihood work item (see bin_loglik_kernel)
 constexpr int BIN_SORT_PER_THREAD = BIN_ITEM / 256;
 constexpr int BIN_MAX_BOX = 128;      // window edge T + 2R (a tensor copy box is at most 256 floats wide)
 
@@ -67,6 +66,14 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
         : "memory");
 }
 
+// bytes (a multiple of 16, both addresses 16-byte aligned) into shared memory, counted on the same barrier
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "l"(src), "r"(bytes), "r"(bar)
+                 : "memory");
+}
+
 // Waits for the phase of the given parity to complete.  Bounded: gives up
 // after about a second of clock cycles (or 2^26 polls) and returns false.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
@@ -89,24 +96,31 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
 
 // ---------------------------------------------------------- the scatter
 // Each block first turns the bin sizes into their exclusive prefix (each
-// bin's first record).  It then takes chunks of BIN_CHUNK consecutive slots,
-// each thread 16 consecutive slots read as 16-byte vectors.  A chunk is
-// ranked by bin in shared memory and staged there in bin order; one global
-// atomic per nonempty bin reserves the chunk's range inside the bin (its
-// cursor), and the staged records are then copied out so that consecutive
+// bin's first record).  It then takes chunks of BIN_CHUNK consecutive slots.
+// A chunk is ranked by bin in shared memory and staged there in bin order; one
+// global atomic per nonempty bin reserves the chunk's range inside the bin
+// (its cursor), and the staged records are then copied out so that consecutive
 // threads write consecutive records of a run.  Each slot's key entry receives
-// its record's place (read by the sums of phase 1).  The last block to finish
-// cuts every bin into work items of at most BIN_ITEM records for the
-// likelihood.
-constexpr int BIN_PER_THREAD = 16;
-constexpr int BIN_CHUNK = 256 * BIN_PER_THREAD;
+// its record's place (read by the sums of phase 1).
+//
+// A chain of latencies bounds it: keys, shared atomics, a prefix, the
+// reservations, staging, each behind a barrier.  So a chunk's keys and states
+// are loaded together at its start, four consecutive slots a lane (coalesced
+// 16-byte vectors), and two blocks of 512 threads share an SM, one grid of
+// resident blocks.  4,000,000 slots, 290 bins: 58.8 us with 16 consecutive
+// slots a thread loaded where they were staged, 33.9 us now (144 MB, 21 us at
+// the copy rate).  Half the chunk doubles the reservations and the runs: 82 us
+// in the first form.
+constexpr int BIN_PER_THREAD = 8;
+constexpr int BIN_QUADS = BIN_PER_THREAD / 4;
+constexpr int BIN_THREADS = 512;
+constexpr int BIN_QSTEP = 4 * BIN_THREADS;
+constexpr int BIN_CHUNK = BIN_THREADS * BIN_PER_THREAD;
 
-__global__ void __launch_bounds__(256) bin_scatter_kernel(const float *__restrict__ st, int64_t N, int nbins,
+__global__ void __launch_bounds__(BIN_THREADS, 2) bin_scatter_kernel(const float *__restrict__ st, int64_t N, int nbins,
                                                           uint32_t *__restrict__ key,
                                                           const uint32_t *__restrict__ size,
-                                                          uint32_t *__restrict__ cursor, float4 *__restrict__ rec,
-                                                          int32_t *__restrict__ items, int items_max,
-                                                          DevSummary *sum)
+                                                          uint32_t *__restrict__ cursor, float4 *__restrict__ rec, DevSummary *sum)
 {
     if (!pdl_wait())
         return;
@@ -139,24 +153,40 @@ __global__ void __launch_bounds__(256) bin_scatter_kernel(const float *__restric
     for (uint32_t lo = blockIdx.x * (uint32_t)BIN_CHUNK; lo < n; lo += gridDim.x * (uint32_t)BIN_CHUNK) {
         for (int t = threadIdx.x; t < nbins; t += blockDim.x)
             cnt[t] = 0u;
-        const uint32_t i0 = lo + threadIdx.x * BIN_PER_THREAD;
-        const bool full = vec_ok && i0 + BIN_PER_THREAD <= n;
+        // quarter q of a thread's slots: four from lo + 4 (q threads + thread)
         uint32_t k[BIN_PER_THREAD], r[BIN_PER_THREAD];
+        float4 xx[BIN_QUADS], yy[BIN_QUADS], zz[BIN_QUADS];
+        const uint32_t i0 = lo + 4u * threadIdx.x;
+        const bool full = vec_ok && n - lo >= (uint32_t)BIN_CHUNK;
         if (full) {
 #pragma unroll
-            for (int q = 0; q < BIN_PER_THREAD / 4; ++q) {
-                const uint4 kk = __ldg(reinterpret_cast<const uint4 *>(key + i0) + q);
+            for (int q = 0; q < BIN_QUADS; ++q) {
+                const uint4 kk = __ldcg(reinterpret_cast<const uint4 *>(key + i0 + q * BIN_QSTEP));
                 k[4 * q] = kk.x; k[4 * q + 1] = kk.y; k[4 * q + 2] = kk.z; k[4 * q + 3] = kk.w;
+            }
+#pragma unroll
+            for (int q = 0; q < BIN_QUADS; ++q) {
+                xx[q] = __ldcg(reinterpret_cast<const float4 *>(st + i0 + q * BIN_QSTEP));
+                yy[q] = __ldcg(reinterpret_cast<const float4 *>(st + N + i0 + q * BIN_QSTEP));
+                zz[q] = __ldcg(reinterpret_cast<const float4 *>(st + 4 * N + i0 + q * BIN_QSTEP));
             }
         } else {
 #pragma unroll
-            for (int e = 0; e < BIN_PER_THREAD; ++e)
-                k[e] = i0 + e < n ? __ldg(key + i0 + e) : 0u;
+            for (int q = 0; q < BIN_QUADS; ++q) {
+                const uint32_t i = i0 + q * BIN_QSTEP;
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    k[4 * q + e] = i + e < n ? __ldcg(key + i + e) : 0u;
+                auto at = [&](const float *p, int e) { return i + e < n ? __ldcg(p + i + e) : 0.0f; };
+                xx[q] = make_float4(at(st, 0), at(st, 1), at(st, 2), at(st, 3));
+                yy[q] = make_float4(at(st + N, 0), at(st + N, 1), at(st + N, 2), at(st + N, 3));
+                zz[q] = make_float4(at(st + 4 * N, 0), at(st + 4 * N, 1), at(st + 4 * N, 2), at(st + 4 * N, 3));
+            }
         }
         __syncthreads();
 #pragma unroll
         for (int e = 0; e < BIN_PER_THREAD; ++e)
-            r[e] = (i0 + e < n) ? atomicAdd(&cnt[k[e]], 1u) : 0u;
+            r[e] = (i0 + (e / 4) * BIN_QSTEP + e % 4 < n) ? atomicAdd(&cnt[k[e]], 1u) : 0u;
         __syncthreads();
         {   // local starts (exclusive prefix of the counts) and the global reservations
             const int per = (nbins + blockDim.x - 1) / blockDim.x, t0 = threadIdx.x * per;
@@ -173,27 +203,15 @@ __global__ void __launch_bounds__(256) bin_scatter_kernel(const float *__restric
             }
         }
         __syncthreads();
-        // stage the records in bin order (the state read now, as 16-byte vectors)
+        // stage the records in bin order
 #pragma unroll
-        for (int q = 0; q < BIN_PER_THREAD / 4; ++q) {
-            float4 xx, yy, zz;
-            if (full) {
-                xx = __ldg(reinterpret_cast<const float4 *>(st + i0) + q);
-                yy = __ldg(reinterpret_cast<const float4 *>(st + N + i0) + q);
-                zz = __ldg(reinterpret_cast<const float4 *>(st + 4 * N + i0) + q);
-            } else {
-                auto at = [&](const float *p, int e) { return i0 + e < n ? __ldg(p + i0 + e) : 0.0f; };
-                xx = make_float4(at(st, 4 * q), at(st, 4 * q + 1), at(st, 4 * q + 2), at(st, 4 * q + 3));
-                yy = make_float4(at(st + N, 4 * q), at(st + N, 4 * q + 1), at(st + N, 4 * q + 2), at(st + N, 4 * q + 3));
-                zz = make_float4(at(st + 4 * N, 4 * q), at(st + 4 * N, 4 * q + 1), at(st + 4 * N, 4 * q + 2),
-                                 at(st + 4 * N, 4 * q + 3));
-            }
-            const float xs[4] = {xx.x, xx.y, xx.z, xx.w}, ys[4] = {yy.x, yy.y, yy.z, yy.w};
-            const float zs[4] = {zz.x, zz.y, zz.z, zz.w};
+        for (int q = 0; q < BIN_QUADS; ++q) {
+            const float xs[4] = {xx[q].x, xx[q].y, xx[q].z, xx[q].w}, ys[4] = {yy[q].x, yy[q].y, yy[q].z, yy[q].w};
+            const float zs[4] = {zz[q].x, zz[q].y, zz[q].z, zz[q].w};
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 const int e = 4 * q + c;
-                if (i0 + e < n) {
+                if (i0 + q * BIN_QSTEP + c < n) {
                     const uint32_t j = lstart[k[e]] + r[e];
                     stage[j] = make_float4(xs[c], ys[c], zs[c], 0.0f);
                     sbin[j] = (uint16_t)k[e];
@@ -203,13 +221,16 @@ __global__ void __launch_bounds__(256) bin_scatter_kernel(const float *__restric
         }
         if (full) {
 #pragma unroll
-            for (int q = 0; q < BIN_PER_THREAD / 4; ++q)
-                reinterpret_cast<uint4 *>(key + i0)[q] = make_uint4(k[4 * q], k[4 * q + 1], k[4 * q + 2], k[4 * q + 3]);
+            for (int q = 0; q < BIN_QUADS; ++q)
+                *reinterpret_cast<uint4 *>(key + i0 + q * BIN_QSTEP) =
+                    make_uint4(k[4 * q], k[4 * q + 1], k[4 * q + 2], k[4 * q + 3]);
         } else {
 #pragma unroll
-            for (int e = 0; e < BIN_PER_THREAD; ++e)
-                if (i0 + e < n)
-                    key[i0 + e] = k[e];
+            for (int e = 0; e < BIN_PER_THREAD; ++e) {
+                const uint32_t i = i0 + (e / 4) * BIN_QSTEP + e % 4;
+                if (i < n)
+                    key[i] = k[e];
+            }
         }
         __syncthreads();
         // copy out: consecutive threads, consecutive records of a bin's run
@@ -222,71 +243,37 @@ __global__ void __launch_bounds__(256) bin_scatter_kernel(const float *__restric
         }
         __syncthreads();
     }
-    // the last block: the likelihood's work items (no block waits for it)
-    __shared__ bool last;
-    if (threadIdx.x == 0) {
-        __threadfence();
-        last = (atomicAdd(&sum->bin_blocks_done, 1u) == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!last)
-        return;
-    __threadfence();
-    uint32_t *sio = reinterpret_cast<uint32_t *>(stage);  // [nbins + 1] item prefix (the stage is free now)
-    {
-        const int per = (nbins + blockDim.x - 1) / blockDim.x, t0 = threadIdx.x * per;
-        uint64_t sm = 0;
-        for (int t = t0; t < t0 + per && t < nbins; ++t)
-            sm += (__ldcg(size + t) + BIN_ITEM - 1) / BIN_ITEM;
-        uint64_t iall;
-        uint64_t run = block_excl_scan_u64(sm, red, &iall);
-        for (int t = t0; t < t0 + per && t < nbins; ++t) {
-            sio[t] = (uint32_t)run;
-            run += (__ldcg(size + t) + BIN_ITEM - 1) / BIN_ITEM;
-        }
-        if (threadIdx.x == 0) {
-            sio[nbins] = (uint32_t)iall;
-            sum->n_bin_items = (int32_t)iall;
-            sum->bin_blocks_done = 0u;
-        }
-    }
-    __syncthreads();
-    const uint32_t ni = sio[nbins];
-    for (uint32_t j = threadIdx.x; j < ni; j += blockDim.x) {
-        int lo = 0, hi = nbins;  // sio[lo] <= j < sio[hi]
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (sio[mid] <= j)
-                lo = mid;
-            else
-                hi = mid;
-        }
-        const uint32_t s0 = (j - sio[lo]) * (uint32_t)BIN_ITEM;
-        const uint32_t sz = __ldcg(size + lo);
-        if (PPF_DCHECK(j < (uint32_t)items_max && s0 < sz, flags, FLAG_INTERNAL)) {
-            items[j] = lo;
-            items[items_max + j] = (int32_t)(bstart[lo] + s0);
-            items[2 * items_max + j] = (int32_t)((sz - s0) < (uint32_t)BIN_ITEM ? (sz - s0) : BIN_ITEM);
-        }
-    }
 }
 
 // ------------------------------------------------------- the likelihood
+// Bound by the shared-memory pipe: a patch at R = 5 takes 66 eight-byte window
+// reads, two wavefronts a warp each, so 4,000,000 records need 56 us of it.
+// What kept the kernel from that was each item's start (its records read from
+// L2 twice around three barriers) and uneven work.  Now the next item's
+// records are copied with its window (one bulk copy each on one barrier)
+// while this item is summed, only the 16-bit order is sorted, a window row is
+// a multiple of 16 pairs (the anchor after the last of a row then stands in
+// the following bank; 254 us instead of 265 for the step), and each block
+// finds its items from the bin sizes, without a list made by the scatter's
+// last block.  Items of 1280 records leave two blocks an SM and deal evenly:
+// the whole binned step of 4,000,000 particles takes 243 us (247 with 1536,
+// 251 with 2048, 262 with 1024; 286 with items of 4096 and none of this), that
+// of 250,000 49 us (66).
 struct BinLikArgs {
     int64_t N;
-    int W, H, T, nx, nbins, box;   // box = T + 2R: window edge in pairs and rows
-    int items_max;
+    int W, H, T, nx, nbins;
+    int box, pitch;                // rows of a window (T + 2R) and pairs in one of its rows (win_pitch)
     int win_stride;                // bytes between the two windows (a multiple of 128)
     float inv2s2, inv_sxi2;
     float Kc[MAX_RADIUS];
     const float4 *__restrict__ rec;
-    const int32_t *__restrict__ items;
+    const uint32_t *__restrict__ size;  // the bin sizes
     float *__restrict__ l;         // l of every record, in bin order
     DevSummary *sum;
 };
 
 template <int R>
-__global__ void __launch_bounds__(256) bin_loglik_kernel(const __grid_constant__ CUtensorMap tmap, BinLikArgs a)
+__global__ void __launch_bounds__(256, 2) bin_loglik_kernel(const __grid_constant__ CUtensorMap tmap, BinLikArgs a)
 {
     if (!pdl_wait())
         return;
@@ -297,62 +284,102 @@ __global__ void __launch_bounds__(256) bin_loglik_kernel(const __grid_constant__
     extern __shared__ __align__(16) unsigned char bsm[];
     __shared__ __align__(8) uint64_t bars[2];
     __shared__ int failed;
-    const int n_items = __ldcg(&sum->n_bin_items);
+    __shared__ uint64_t red[33];
     // the windows start on a 128-byte boundary (the launch adds 128 bytes of
-    // slack); then the item's records sorted by anchor and the anchor counts
+    // slack); then two items' records, the current item's order by anchor,
+    // the anchor counts, and the bins' first records and items
     const uint32_t base = smem_u32(bsm), pad = ((base + 127u) & ~127u) - base;
     unsigned char *wbase = bsm + pad;
-    float4 *srt = reinterpret_cast<float4 *>(wbase + 2 * a.win_stride);
+    float4 *raw = reinterpret_cast<float4 *>(wbase + 2 * a.win_stride);
+    uint16_t *srt = reinterpret_cast<uint16_t *>(raw + 2 * BIN_ITEM);
     uint32_t *hist = reinterpret_cast<uint32_t *>(srt + BIN_ITEM);
-    __shared__ uint64_t red[33];
+    uint32_t *bs = hist + a.T * a.T, *is = bs + a.nbins + 1;
     const uint32_t bar0 = smem_u32(&bars[0]), bar1 = smem_u32(&bars[1]);
-    const uint32_t win0 = base + pad, win1 = win0 + (uint32_t)a.win_stride;
-    const uint32_t box_bytes = (uint32_t)(a.box * a.box * 8);
+    const uint32_t win0 = base + pad, win1 = win0 + (uint32_t)a.win_stride, raw0 = smem_u32(raw);
+    const uint32_t box_bytes = (uint32_t)(a.box * a.pitch * 8);
     if (threadIdx.x == 0) {
         mbar_init(bar0);
         mbar_init(bar1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         failed = 0;
     }
+    int n_items;
+    {   // first item and first record of every bin
+        const int per = (a.nbins + blockDim.x - 1) / blockDim.x, t0 = threadIdx.x * per;
+        uint64_t sm = 0;
+        for (int t = t0; t < t0 + per && t < a.nbins; ++t) {
+            const uint32_t z = __ldcg(a.size + t);
+            sm += ((uint64_t)((z + BIN_ITEM - 1) / BIN_ITEM) << 32) + z;
+        }
+        uint64_t all;
+        uint64_t run = block_excl_scan_u64(sm, red, &all);
+        for (int t = t0; t < t0 + per && t < a.nbins; ++t) {
+            const uint32_t z = __ldcg(a.size + t);
+            bs[t] = (uint32_t)run;
+            is[t] = (uint32_t)(run >> 32);
+            run += ((uint64_t)((z + BIN_ITEM - 1) / BIN_ITEM) << 32) + z;
+        }
+        n_items = (int)(all >> 32);
+        if (threadIdx.x == 0) {
+            bs[a.nbins] = (uint32_t)all;
+            is[a.nbins] = (uint32_t)n_items;
+        }
+    }
     __syncthreads();
-    const int32_t *ibin = a.items, *istart = a.items + a.items_max, *icount = a.items + 2 * a.items_max;
+    struct Item {
+        int t;
+        uint32_t s0, cnt;
+    };
+    auto item_at = [&](int j) -> Item {  // j < n_items
+        int lo = 0, up = a.nbins;        // is[lo] <= j < is[up]
+        while (up - lo > 1) {
+            const int mid = (lo + up) >> 1;
+            if (is[mid] <= (uint32_t)j)
+                lo = mid;
+            else
+                up = mid;
+        }
+        const uint32_t s0 = bs[lo] + ((uint32_t)j - is[lo]) * (uint32_t)BIN_ITEM;
+        return Item{lo, s0, min(bs[lo + 1] - s0, (uint32_t)BIN_ITEM)};
+    };
     const int special = a.nbins - 1;
-    auto issue = [&](int j, int buf) {  // thread 0: the window of item j into buffer buf
-        const int t = __ldg(ibin + j);
-        if (t == special)
+    auto issue = [&](const Item &it, int buf) {  // thread 0: the item's window and records into buffer buf
+        if (it.t == special)
             return;
-        const int tx = t % a.nx, ty = t / a.nx;
+        const int tx = it.t % a.nx, ty = it.t / a.nx;
         const uint32_t bar = buf ? bar1 : bar0;
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        mbar_expect_tx(bar, box_bytes);
+        mbar_expect_tx(bar, box_bytes + 16u * it.cnt);
         tma_load_2d(buf ? win1 : win0, &tmap, 2 * tx * a.T, ty * a.T, bar);
+        bulk_load(raw0 + (buf ? 16u * (uint32_t)BIN_ITEM : 0u), a.rec + it.s0, 16u * it.cnt, bar);
     };
     const PatchGeom geom{nullptr, a.W, a.H, 0, 0, a.inv2s2, a.inv_sxi2, a.Kc, 0, &sum->flags};
     const float4 *__restrict__ rec = a.rec;
-    // Thread 0 issues every window copy; all threads wait on its barrier.  A
-    // wait that times out stops the block's work (the flag reports it), and
+    // Thread 0 issues every copy; all threads wait on its barrier.  A wait
+    // that times out stops the block's work (the flag reports it), and
     // thread 0 then waits once more, bounded, for the copies it left in
     // flight before the block's shared memory is released.
     // bit b of phase: the parity of buffer b's next copy; bit b of pend: a
     // copy into buffer b issued and not yet waited for
     uint32_t phase = 0u, pend = 0u;
     int k = 0;
-    if ((int)blockIdx.x < n_items) {
-        if (threadIdx.x == 0)
-            issue(blockIdx.x, 0);
-        pend |= (__ldg(ibin + blockIdx.x) != special) ? 1u : 0u;
-    }
+    if ((int)blockIdx.x >= n_items)
+        return;
+    Item next = item_at(blockIdx.x);
+    if (threadIdx.x == 0)
+        issue(next, 0);
+    pend |= (next.t != special) ? 1u : 0u;
     for (int j = blockIdx.x; j < n_items; j += gridDim.x, ++k) {
         const int buf = k & 1;
-        const int jn = j + (int)gridDim.x;
-        if (jn < n_items) {  // the next item's window, copied while this one is summed
+        const int t = next.t;
+        const int s0 = (int)next.s0, cntj = (int)next.cnt;
+        if (j + (int)gridDim.x < n_items) {  // the next item's copies run while this one is summed
+            next = item_at(j + (int)gridDim.x);
             if (threadIdx.x == 0)
-                issue(jn, buf ^ 1);
-            if (__ldg(ibin + jn) != special)
+                issue(next, buf ^ 1);
+            if (next.t != special)
                 pend |= 1u << (buf ^ 1);
         }
-        const int t = __ldg(ibin + j);
-        const int s0 = __ldg(istart + j), cntj = __ldg(icount + j);
         if (t != special) {
             if (mbar_wait(buf ? bar1 : bar0, (phase >> buf) & 1u)) {
                 phase ^= 1u << buf;
@@ -366,6 +393,7 @@ __global__ void __launch_bounds__(256) bin_loglik_kernel(const __grid_constant__
                 break;
         }
         const float2 *win = reinterpret_cast<const float2 *>(wbase + (buf ? a.win_stride : 0));
+        const float4 *rb = raw + (buf ? BIN_ITEM : 0);
         const int tx = t % a.nx, ty = t / a.nx;
         constexpr int P = 2 * R + 1;
         if (t == special) {  // no patch sums: l = -inf (non-finite) or 0 (no pixel in the image)
@@ -384,17 +412,17 @@ __global__ void __launch_bounds__(256) bin_loglik_kernel(const __grid_constant__
             for (int u = threadIdx.x; u < a.T * a.T; u += blockDim.x)
                 hist[u] = 0u;
             __syncthreads();
-            uint32_t an[BIN_SORT_PER_THREAD], rk[BIN_SORT_PER_THREAD];
+            uint32_t an[BIN_SORT_PER_THREAD];  // anchor and rank
 #pragma unroll
             for (int e = 0; e < BIN_SORT_PER_THREAD; ++e) {
                 const int r = threadIdx.x + e * (int)blockDim.x;
-                const float2 xy = r < cntj ? *reinterpret_cast<const float2 *>(rec + s0 + r) : make_float2(0.0f, 0.0f);
+                const float2 xy = r < cntj ? *reinterpret_cast<const float2 *>(rb + r) : make_float2(0.0f, 0.0f);
                 const int lu = (int)floorf(xy.x + 0.5f) + R - tx * a.T;
                 const int lv = (int)floorf(xy.y + 0.5f) + R - ty * a.T;
                 const bool ok = r < cntj && PPF_DCHECK(lu >= 0 && lu < a.T && lv >= 0 && lv < a.T, &sum->flags,
                                                        FLAG_INTERNAL);
-                an[e] = ok ? (uint32_t)(lv * a.T + lu) : 0xFFFFFFFFu;
-                rk[e] = ok ? atomicAdd(&hist[an[e]], 1u) : 0u;
+                const uint32_t u = (uint32_t)(lv * a.T + lu);
+                an[e] = ok ? u | (atomicAdd(&hist[u], 1u) << 16) : 0xFFFFFFFFu;
             }
             __syncthreads();
             // exclusive prefix of the T x T counts (at most 4096: 16 per thread)
@@ -414,22 +442,20 @@ __global__ void __launch_bounds__(256) bin_loglik_kernel(const __grid_constant__
             __syncthreads();
 #pragma unroll
             for (int e = 0; e < BIN_SORT_PER_THREAD; ++e)
-                if (an[e] != 0xFFFFFFFFu) {  // the record again (from L2), to its sorted place
-                    const int r = threadIdx.x + e * (int)blockDim.x;
-                    const float4 q = rec[s0 + r];
-                    srt[hist[an[e]] + rk[e]] = make_float4(q.x, q.y, q.z, __uint_as_float((uint32_t)r));
-                }
+                if (an[e] != 0xFFFFFFFFu)
+                    srt[hist[an[e] & 0xFFFFu] + (an[e] >> 16)] = (uint16_t)(threadIdx.x + e * blockDim.x);
             __syncthreads();
             for (int j = threadIdx.x; j < cntj; j += blockDim.x) {
-                const float4 v = srt[j];  // (x, y, I0, the record's place in the item)
+                const uint32_t r = srt[j];
+                const float4 v = rb[r];
                 int cx, cy;
                 float gx[P], gy[P], C, l;
                 if (patch_setup<R>(geom, v.x, v.y, v.z, cx, cy, gx, gy, C, &l)) {
                     const int lu = cx + R - tx * a.T, lv = cy + R - ty * a.T;
-                    const float Bs = patch_rows<R, true, true>(win + lv * a.box + lu, a.box, gx, gy);
+                    const float Bs = patch_rows<R, true, true>(win + lv * a.pitch + lu, a.pitch, gx, gy);
                     l = v.z * fmaf(-0.5f * v.z, C, Bs) * a.inv_sxi2;
                 }
-                a.l[s0 + __float_as_uint(v.w)] = l;
+                a.l[s0 + r] = l;
             }
         }
         __syncthreads();  // this window is free for the copy two items on
@@ -445,9 +471,12 @@ __global__ void __launch_bounds__(256) bin_loglik_kernel(const __grid_constant__
 // ------------------------------------------------------------ host side
 namespace {
 
+// pairs in a row of the window: whole turns of the 32 banks (see bin_loglik_kernel)
+int win_pitch(int box) { return (box + 15) / 16 * 16; }
+
 int win_stride_bytes(int box)
 {
-    const int b = box * box * 8;
+    const int b = box * win_pitch(box) * 8;
     return (b + 127) / 128 * 128;
 }
 
@@ -457,10 +486,11 @@ size_t scatter_smem(int nbins)
     return sizeof(float4) * BIN_CHUNK + sizeof(uint16_t) * BIN_CHUNK + 4 * sizeof(uint32_t) * (size_t)nbins;
 }
 
-size_t loglik_smem(int box, int T)
+size_t loglik_smem(int box, int T, int nbins)
 {
-    // two windows, the alignment slack, the sorted records, the anchor counts
-    return 2 * (size_t)win_stride_bytes(box) + 128 + sizeof(float4) * BIN_ITEM + sizeof(uint32_t) * T * T;
+    // two windows, the alignment slack, two items' records and their order, the anchor counts, the bin prefixes
+    return 2 * (size_t)win_stride_bytes(box) + 128 + (2 * sizeof(float4) + sizeof(uint16_t)) * BIN_ITEM +
+           sizeof(uint32_t) * (T * T + 2 * ((size_t)nbins + 1));
 }
 
 // The dynamic shared memory limit of a kernel is raised to the device's
@@ -536,25 +566,26 @@ cudaError_t bin_setup(ppf_ctx *c)
     c->bin_T = T;
     c->bin_nx = (c->m.width + 2 * R + T - 1) / T;
     c->bin_nbins = (int32_t)bins(T);
-    c->bin_items_max = c->bin_nbins + (int32_t)((c->N + BIN_ITEM - 1) / BIN_ITEM);
     const int box = T + 2 * R;
-    const size_t smem = loglik_smem(box, T);
+    const size_t smem = loglik_smem(box, T, c->bin_nbins);
     int per_sm = 0;
     cudaError_t e = loglik_setup(R, smem, &per_sm);
     if (e != cudaSuccess)
         return e;
     c->bin_grid = c->num_sms * (per_sm > 0 ? (per_sm < 4 ? per_sm : 4) : 1);
     e = raise_smem_limit(bin_scatter_kernel, scatter_smem(c->bin_nbins));
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bin_scatter_kernel, BIN_THREADS, scatter_smem(c->bin_nbins));
     if (e != cudaSuccess)
         return e;
+    c->bin_scatter_grid = c->num_sms * (per_sm > 0 ? per_sm : 1);
     if ((e = dalloc(&c->bin_key, (size_t)c->N)) != cudaSuccess ||
         (e = dalloc(&c->bin_l, (size_t)c->N)) != cudaSuccess ||
         (e = dalloc(&c->bin_tot, 2 * ((size_t)c->bin_nbins + 1))) != cudaSuccess ||
-        (e = dalloc(&c->bin_item, 3 * (size_t)c->bin_items_max)) != cudaSuccess ||
         (e = dalloc(&c->bin_rec, (size_t)c->N)) != cudaSuccess)
         return e;
     // the prepared frame as a 2D float tensor (2 Wp floats per row, Hp rows);
-    // a window is 2 box floats by box rows, copied with zero fill outside
+    // a window is 2 win_pitch(box) floats by box rows, copied with zero fill outside
     void *fn = nullptr;
     cudaDriverEntryPointQueryResult q;
     e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q);
@@ -562,7 +593,7 @@ cudaError_t bin_setup(ppf_ctx *c)
         return e != cudaSuccess ? e : cudaErrorNotSupported;
     const cuuint64_t dims[2] = {(cuuint64_t)2 * c->Wp, (cuuint64_t)c->Hp};
     const cuuint64_t strides[1] = {(cuuint64_t)2 * c->Wp * sizeof(float)};
-    const cuuint32_t boxd[2] = {(cuuint32_t)(2 * box), (cuuint32_t)box};
+    const cuuint32_t boxd[2] = {(cuuint32_t)(2 * win_pitch(box)), (cuuint32_t)box};
     const cuuint32_t estr[2] = {1, 1};
     const CUresult r = reinterpret_cast<EncodeTiled>(fn)(
         &c->bin_tmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, c->Zp, dims, strides, boxd, estr,
@@ -595,9 +626,9 @@ cudaError_t launch_binned(ppf_ctx *c)
     const int nb = c->bin_nbins;
     float *dst = c->state[c->cur ^ 1];
     const int64_t chunks = (c->N + BIN_CHUNK - 1) / BIN_CHUNK;
-    const int gscat = (int)(chunks < 4 * (int64_t)c->num_sms ? chunks : 4 * (int64_t)c->num_sms);
-    launch_pdl(bin_scatter_kernel, gscat, 256, scatter_smem(nb), c->stream, (const float *)dst, c->N, nb, c->bin_key,
-               (const uint32_t *)c->bin_tot, c->bin_tot + nb + 1, c->bin_rec, c->bin_item, c->bin_items_max, c->sum);
+    const int gscat = (int)(chunks < (int64_t)c->bin_scatter_grid ? chunks : (int64_t)c->bin_scatter_grid);
+    launch_pdl(bin_scatter_kernel, gscat, BIN_THREADS, scatter_smem(nb), c->stream, (const float *)dst, c->N, nb, c->bin_key,
+               (const uint32_t *)c->bin_tot, c->bin_tot + nb + 1, c->bin_rec, c->sum);
     BinLikArgs a;
     memset(&a, 0, sizeof(a));
     a.N = c->N;
@@ -607,17 +638,17 @@ cudaError_t launch_binned(ppf_ctx *c)
     a.nx = c->bin_nx;
     a.nbins = nb;
     a.box = c->bin_T + 2 * R;
-    a.items_max = c->bin_items_max;
+    a.pitch = win_pitch(a.box);
     a.win_stride = win_stride_bytes(a.box);
     a.inv2s2 = 1.0f / (2.0f * c->m.psf_sigma * c->m.psf_sigma);
     a.inv_sxi2 = 1.0f / (c->m.sigma_xi * c->m.sigma_xi);
     for (int q = 0; q < MAX_RADIUS; ++q)
         a.Kc[q] = (float)exp(-(2.0 * q + 1.0) * (double)a.inv2s2);
     a.rec = c->bin_rec;
-    a.items = c->bin_item;
+    a.size = c->bin_tot;
     a.l = c->bin_l;
     a.sum = c->sum;
-    const size_t smem = loglik_smem(a.box, a.T);
+    const size_t smem = loglik_smem(a.box, a.T, nb);
     switch (R) {
     case 0: launch_loglik_r<0>(c->bin_tmap, a, c->bin_grid, smem, c->stream); break;
     case 1: launch_loglik_r<1>(c->bin_tmap, a, c->bin_grid, smem, c->stream); break;

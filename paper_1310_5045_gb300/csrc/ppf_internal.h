@@ -99,8 +99,6 @@ struct DevSummary {
     // decided by the step's finaliser from the warps it saw spread
     int32_t bin_this, bin_next;
     uint32_t spread_warps, total_warps;
-    uint32_t bin_blocks_done;  // binned path: scatter blocks that finished
-    int32_t n_bin_items;       // binned path: likelihood work items of this step
     int32_t n_split;           // two-stage RPA: extra work items of large or heavy groups (group_grid_kernel)
     int32_t n_runs;            // and the further runs of heavy tile parts, listed after them (split_runs_kernel)
     int32_t n_extra;           // the fill's further runs of ticket-heavy tiles (tile_tickets_kernel)
@@ -185,11 +183,11 @@ struct ppf_ctx {
     ppf::Scratch sc;
     // binned likelihood path (input-space decomposition): tiles of bin_T
     // anchors, bin_nbins bins (the last for particles with no patch sum)
-    int32_t bin_T, bin_nx, bin_nbins, bin_grid, bin_items_max;  // bin_grid: blocks of the binned likelihood
+    int32_t bin_T, bin_nx, bin_nbins;
+    int32_t bin_grid, bin_scatter_grid;  // blocks of the binned likelihood and of the scatter at most
     int bin_force;                // -1: chosen per step on the device; 0: direct path; 1: binned path
     uint32_t *bin_key;            // [N] bin of every slot, then the place of its record in bin order
     uint32_t *bin_tot;            // [2 (nbins + 1)] bin sizes, then the scatter's cursors (offsets inside each bin)
-    int32_t *bin_item;            // [3 x items_max] work items: bin, first record, count
     float4 *bin_rec;              // [N] records in bin order: (x, y, I0, -)
     float *bin_l;                 // [N] l of every record, in bin order
     CUtensorMap bin_tmap;         // the prepared frame as a 2D float tensor for the window copies (64-byte aligned type)
@@ -247,6 +245,7 @@ cudaError_t launch_draw_plain(const float *lw, int64_t N, DevSummary *sum, uint6
                               int64_t *Tt, int32_t *To, int2 *extra, uint64_t seed, uint32_t fid, uint32_t frame,
                               int32_t *out, cudaStream_t stream);
 cudaError_t launch_identity(ppf_ctx *c, int32_t *dst);
+cudaError_t launch_restart(ppf_ctx *c, bool identity);
 cudaError_t launch_pending(ppf_ctx *c, int32_t *anc_out, float *lwp_out);
 cudaError_t launch_fill_f32(ppf_ctx *c, float *dst, float v);
 cudaError_t launch_format_estimate(ppf_ctx *c, ppf_estimate_t *out);

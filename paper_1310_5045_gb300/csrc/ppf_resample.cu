@@ -2212,6 +2212,31 @@ __global__ void identity_kernel(int32_t *__restrict__ a, int64_t N)
         a[i] = (int32_t)i;
 }
 
+// New particles were set: identity ancestry (a non-null), no degenerate
+// resample before them, and the binned path next if the context has it.
+// One launch for what were an ancestor fill and two copies of four bytes from
+// the host, each staged and one of them waited for.
+__global__ void restart_kernel(int32_t *__restrict__ a, int64_t N, DevSummary *sum, int binned)
+{
+    if (!pdl_wait())
+        return;
+    pdl_trigger();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        sum->degenerate = 0;
+        if (binned)
+            sum->bin_next = 1;
+    }
+    if (!a)
+        return;
+    const int64_t nv = N >> 2;
+    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < nv; v += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t i = (int32_t)(4 * v);
+        reinterpret_cast<int4 *>(a)[v] = make_int4(i, i + 1, i + 2, i + 3);
+    }
+    if (blockIdx.x == 0 && threadIdx.x < (N & 3))
+        a[4 * nv + threadIdx.x] = (int32_t)(4 * nv + threadIdx.x);
+}
+
 __global__ void fill_f32_kernel(float *__restrict__ a, int64_t N, float v)
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
@@ -2420,6 +2445,15 @@ cudaError_t launch_identity(ppf_ctx *c, int32_t *dst)
     const int grid = (int)((c->N + 255) / 256 < 8192 ? (c->N + 255) / 256 : 8192);
     c->launches += 1;
     identity_kernel<<<grid, 256, 0, c->stream>>>(dst, c->N);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_restart(ppf_ctx *c, bool identity)
+{
+    const int64_t need = identity ? (c->N / 4 + 255) / 256 + 1 : 1;
+    const int grid = (int)(need < 8 * (int64_t)c->num_sms ? need : 8 * (int64_t)c->num_sms);
+    c->launches += 1;
+    launch_pdl(restart_kernel, grid, 256, 0, c->stream, identity ? c->anc : nullptr, c->N, c->sum, c->bin_key ? 1 : 0);
     return cudaGetLastError();
 }
 
