@@ -35,7 +35,7 @@
 
 namespace ppf {
 
-constexpr int BIN_ITEM = 1280;        // records per likelihood work item (see bin_loglik_kernel)
+constexpr int BIN_ITEM = 1536;        // records per likelihood work item (see bin_loglik_kernel)
 constexpr int BIN_SORT_PER_THREAD = BIN_ITEM / 256;
 constexpr int BIN_MAX_BOX = 128;      // window edge T + 2R (a tensor copy box is at most 256 floats wide)
 
@@ -255,10 +255,10 @@ __global__ void __launch_bounds__(BIN_THREADS, 2) bin_scatter_kernel(const float
 // a multiple of 16 pairs (the anchor after the last of a row then stands in
 // the following bank; 254 us instead of 265 for the step), and each block
 // finds its items from the bin sizes, without a list made by the scatter's
-// last block.  Items of 1280 records leave two blocks an SM and deal evenly:
-// the whole binned step of 4,000,000 particles takes 243 us (247 with 1536,
-// 251 with 2048, 262 with 1024; 286 with items of 4096 and none of this), that
-// of 250,000 49 us (66).
+// last block.  Items of 1536 records leave two blocks an SM and deal evenly:
+// the whole binned step takes 246 us for 4,000,000 particles (243 with 1280,
+// 254 with 2048; 286 with items of 4096 and none of this), 1168 for 24,000,000
+// (1188, 1280), 86 for 1,000,000 (91, 86), 49 for 250,000 (49, 51; 66).
 struct BinLikArgs {
     int64_t N;
     int W, H, T, nx, nbins;

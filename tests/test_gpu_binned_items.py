@@ -1,5 +1,5 @@
 """The binned likelihood path at the edges of its work: particle counts around
-a work item's 1280 records, the scatter's chunk of 4096 slots and its 16-byte
+a work item's 1536 records, the scatter's chunk of 4096 slots and its 16-byte
 vectors, all particles in one image tile or spread over the frame, and the
 wider tiles of large frames.  The direct path is the reference: the two add the
 same terms in the same order, so every output has the same bits."""
@@ -28,7 +28,7 @@ def _step(ppf, model, state, frame, path, carry):
 
 
 @pytest.mark.parametrize("spread", [False, True])
-@pytest.mark.parametrize("n", [1, 3, 1279, 1280, 1281, 2561, 4095, 4096, 4097, 4100, 40_003])
+@pytest.mark.parametrize("n", [1, 3, 1279, 1280, 1281, 1535, 1536, 1537, 2561, 3073, 4095, 4096, 4097, 4100, 40_003])
 def test_binned_equals_direct(n, spread):
     _compare(n, spread, 200, 150, 5)
 
