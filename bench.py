@@ -39,7 +39,7 @@ STEP_BYTES = 48
 # measured DRAM bytes per particle of the same kernel (ncu dram__bytes_read.sum +
 # dram__bytes_write.sum, the 5th launch at N = 16M, the step kernel's summary under
 # profiles/), scaled to a launch by N; set to None whenever step_kernel changes
-STEP_TRAFFIC_PER_PARTICLE = (347167744 + 338496768) / 16e6
+STEP_TRAFFIC_PER_PARTICLE = (347141120 + 338872576) / 16e6
 # algorithmic FP32 flops per particle of the likelihood + propagation (an FMA
 # counts 2), two counts:
 #  * the expanded form the kernel evaluates, l = I0 (B - I0 C / 2) / sigma_xi^2
