@@ -185,9 +185,11 @@ ppf_status ppf_resample_if(ppf_ctx *ctx, ppf_scheme scheme, float exchange_ratio
 ppf_status ppf_estimate(ppf_ctx *ctx, ppf_estimate_t *out);
 
 /* ppf_estimate without waiting: enqueues, on the context's stream, a copy of
- * the same fields into out_host and returns.  out_host must be host memory
- * the device can write (page-locked or registered) and must stay valid until
- * the stream has run the copy; read it after synchronising the stream.  The
+ * the same fields into out_host and returns.  out_host must be host memory, at
+ * any address, and must stay valid until the stream has run the copy; read it
+ * after synchronising the stream.  Page-locked (or registered) memory on an
+ * 8-byte boundary is written by the kernel itself; any other address gets a
+ * staged copy, which in pageable memory may make the call wait.  The
  * device flags are reported in status_flags but not cleared (ppf_estimate
  * clears them).  This lets a caller read every frame's result while the
  * next frames are already queued.

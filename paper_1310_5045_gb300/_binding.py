@@ -317,11 +317,15 @@ class ParticleFilter:
 
     def estimate_async(self, out=None):
         """Enqueue a copy of the estimate into `out` (a page-locked uint8
-        tensor of the estimate's size, made when None) and return it without
-        waiting; decode with Estimate.from_buffer once the stream has run."""
+        tensor of the estimate's size, made when None; a slice of a larger one
+        may start at any byte) and return it without waiting; decode with
+        Estimate.from_buffer once the stream has run."""
         torch = self._torch
+        size = C.sizeof(_Estimate)
         if out is None:
-            out = torch.empty(C.sizeof(_Estimate), dtype=torch.uint8, pin_memory=True)
+            out = torch.empty(size, dtype=torch.uint8, pin_memory=True)
+        elif not out.is_contiguous() or out.numel() * out.element_size() < size:
+            raise ValueError(f"out must be a contiguous tensor of at least {size} bytes")
         self._check(self.L.ppf_estimate_async(self._ctx, C.c_void_p(out.data_ptr())), "ppf_estimate_async")
         return out
 

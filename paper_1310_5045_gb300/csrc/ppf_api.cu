@@ -9,6 +9,7 @@
 
 #include "ppf_device.cuh"
 #include "ppf_internal.h"
+#include "ppf_mapped.h"
 
 using namespace ppf;
 
@@ -454,13 +455,18 @@ ppf_status ppf_estimate_async(ppf_ctx *c, ppf_estimate_t *out)
         return PPF_EINVAL;
     if (!c->stepped)
         return PPF_ESTATE;
-    // the kernel writes the caller's page-locked buffer itself where the device
-    // can address it (one launch and no copy); otherwise a staged copy
-    void *dev = nullptr;
-    if (cudaHostGetDevicePointer(&dev, out, 0) == cudaSuccess && dev) {
-        CK(ppf::launch_format_estimate(c, (ppf_estimate_t *)dev));
-    } else {
+    // the kernel writes the caller's page-locked buffer itself where it may (one
+    // launch and no copy); otherwise a staged copy, which takes any host address
+    auto map = [](void *p) -> void * {
+        void *d = nullptr;
+        if (cudaHostGetDevicePointer(&d, p, 0) == cudaSuccess)
+            return d;
         cudaGetLastError();
+        return nullptr;
+    };
+    if (void *dev = ppf::mapped_words(out, sizeof(ppf_estimate_t), map)) {
+        CK(ppf::launch_format_estimate(c, static_cast<ppf_estimate_t *>(dev)));
+    } else {
         CK(ppf::launch_format_estimate(c, c->est_dev));
         CK(cudaMemcpyAsync(out, c->est_dev, sizeof(ppf_estimate_t), cudaMemcpyDeviceToHost, c->stream));
     }
