@@ -35,8 +35,11 @@
 
 namespace ppf {
 
-constexpr int BIN_ITEM = 1536;        // records per likelihood work item (see bin_loglik_kernel)
-constexpr int BIN_SORT_PER_THREAD = BIN_ITEM / 256;
+// records per likelihood work item and threads of its block (see bin_loglik_kernel); WIDE: tiles of more than 32 anchors
+template <bool WIDE>
+struct BinShape {
+    static constexpr int THREADS = WIDE ? 512 : 256, ITEM = WIDE ? 2560 : 1536, BLOCKS = WIDE ? 1 : 2;
+};
 constexpr int BIN_MAX_BOX = 128;      // window edge T + 2R (a tensor copy box is at most 256 floats wide)
 
 // ---------------------------------------------------------- PTX helpers
@@ -259,6 +262,16 @@ __global__ void __launch_bounds__(BIN_THREADS, 2) bin_scatter_kernel(const float
 // the whole binned step takes 246 us for 4,000,000 particles (243 with 1280,
 // 254 with 2048; 286 with items of 4096 and none of this), 1168 for 24,000,000
 // (1188, 1280), 86 for 1,000,000 (91, 86), 49 for 250,000 (49, 51; 66).
+//
+// Tiles of 64 anchors (frames of more than 3072 tiles of 32): an item's window
+// of up to 51 KB and its 4096 anchor counts leave room for one block an SM and
+// cost every item more, so the block has 512 threads and items of 2560
+// records, the most that fits at R = 8.  Particles set over the whole frame
+// and stepped, with this, with 256 threads and 1536, and as it was before the
+// records were copied ahead (256, 4096): 8,000,000 on 3500 x 3000 at R = 8
+// 1237, 1417, 1271 us; on 2200 x 2200 at R = 5 758, 874, 862 us; 4,000,000
+// there 453, 515, 491 us; 50,000 108, 121, 150 us.  (512 threads and 2048: 1361,
+// 752, 426, 105; 256 and 2560: 1308, 809, 488, 122.)
 struct BinLikArgs {
     int64_t N;
     int W, H, T, nx, nbins;
@@ -272,9 +285,11 @@ struct BinLikArgs {
     DevSummary *sum;
 };
 
-template <int R>
-__global__ void __launch_bounds__(256, 2) bin_loglik_kernel(const __grid_constant__ CUtensorMap tmap, BinLikArgs a)
+template <int R, bool WIDE>
+__global__ void __launch_bounds__(BinShape<WIDE>::THREADS, BinShape<WIDE>::BLOCKS)
+    bin_loglik_kernel(const __grid_constant__ CUtensorMap tmap, BinLikArgs a)
 {
+    constexpr int BIN_ITEM = BinShape<WIDE>::ITEM, BIN_SORT_PER_THREAD = BIN_ITEM / BinShape<WIDE>::THREADS;
     if (!pdl_wait())
         return;
     pdl_trigger();
@@ -425,7 +440,7 @@ __global__ void __launch_bounds__(256, 2) bin_loglik_kernel(const __grid_constan
                 an[e] = ok ? u | (atomicAdd(&hist[u], 1u) << 16) : 0xFFFFFFFFu;
             }
             __syncthreads();
-            // exclusive prefix of the T x T counts (at most 4096: 16 per thread)
+            // exclusive prefix of the T x T counts
             {
                 const int na = a.T * a.T, per = (na + blockDim.x - 1) / blockDim.x, u0 = threadIdx.x * per;
                 uint64_t sm = 0;
@@ -486,10 +501,13 @@ size_t scatter_smem(int nbins)
     return sizeof(float4) * BIN_CHUNK + sizeof(uint16_t) * BIN_CHUNK + 4 * sizeof(uint32_t) * (size_t)nbins;
 }
 
+bool wide_tiles(int T) { return T > 32; }
+
 size_t loglik_smem(int box, int T, int nbins)
 {
+    const size_t item = wide_tiles(T) ? BinShape<true>::ITEM : BinShape<false>::ITEM;
     // two windows, the alignment slack, two items' records and their order, the anchor counts, the bin prefixes
-    return 2 * (size_t)win_stride_bytes(box) + 128 + (2 * sizeof(float4) + sizeof(uint16_t)) * BIN_ITEM +
+    return 2 * (size_t)win_stride_bytes(box) + 128 + (2 * sizeof(float4) + sizeof(uint16_t)) * item +
            sizeof(uint32_t) * (T * T + 2 * ((size_t)nbins + 1));
 }
 
@@ -515,27 +533,29 @@ cudaError_t raise_smem_limit(K kernel, size_t need)
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
 }
 
-template <int R>
+template <int R, bool WIDE>
 cudaError_t loglik_attr(size_t smem, int *per_sm)
 {
-    cudaError_t e = raise_smem_limit(bin_loglik_kernel<R>, smem);
+    cudaError_t e = raise_smem_limit(bin_loglik_kernel<R, WIDE>, smem);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, bin_loglik_kernel<R>, 256, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, bin_loglik_kernel<R, WIDE>, BinShape<WIDE>::THREADS,
+                                                          smem);
     return e;
 }
 
+template <bool WIDE>
 cudaError_t loglik_setup(int R, size_t smem, int *per_sm)
 {
     switch (R) {
-    case 0: return loglik_attr<0>(smem, per_sm);
-    case 1: return loglik_attr<1>(smem, per_sm);
-    case 2: return loglik_attr<2>(smem, per_sm);
-    case 3: return loglik_attr<3>(smem, per_sm);
-    case 4: return loglik_attr<4>(smem, per_sm);
-    case 5: return loglik_attr<5>(smem, per_sm);
-    case 6: return loglik_attr<6>(smem, per_sm);
-    case 7: return loglik_attr<7>(smem, per_sm);
-    default: return loglik_attr<8>(smem, per_sm);
+    case 0: return loglik_attr<0, WIDE>(smem, per_sm);
+    case 1: return loglik_attr<1, WIDE>(smem, per_sm);
+    case 2: return loglik_attr<2, WIDE>(smem, per_sm);
+    case 3: return loglik_attr<3, WIDE>(smem, per_sm);
+    case 4: return loglik_attr<4, WIDE>(smem, per_sm);
+    case 5: return loglik_attr<5, WIDE>(smem, per_sm);
+    case 6: return loglik_attr<6, WIDE>(smem, per_sm);
+    case 7: return loglik_attr<7, WIDE>(smem, per_sm);
+    default: return loglik_attr<8, WIDE>(smem, per_sm);
     }
 }
 
@@ -569,7 +589,7 @@ cudaError_t bin_setup(ppf_ctx *c)
     const int box = T + 2 * R;
     const size_t smem = loglik_smem(box, T, c->bin_nbins);
     int per_sm = 0;
-    cudaError_t e = loglik_setup(R, smem, &per_sm);
+    cudaError_t e = wide_tiles(T) ? loglik_setup<true>(R, smem, &per_sm) : loglik_setup<false>(R, smem, &per_sm);
     if (e != cudaSuccess)
         return e;
     c->bin_grid = c->num_sms * (per_sm > 0 ? (per_sm < 4 ? per_sm : 4) : 1);
@@ -617,7 +637,10 @@ cudaError_t bin_set_next(ppf_ctx *c, int binned)
 template <int R>
 static void launch_loglik_r(const CUtensorMap &tm, const BinLikArgs &a, int grid, size_t smem, cudaStream_t s)
 {
-    launch_pdl(bin_loglik_kernel<R>, grid, 256, smem, s, tm, a);
+    if (wide_tiles(a.T))
+        launch_pdl(bin_loglik_kernel<R, true>, grid, BinShape<true>::THREADS, smem, s, tm, a);
+    else
+        launch_pdl(bin_loglik_kernel<R, false>, grid, BinShape<false>::THREADS, smem, s, tm, a);
 }
 
 cudaError_t launch_binned(ppf_ctx *c)
