@@ -6,6 +6,7 @@
 #include <cuda_fp16.h>
 
 #include <cmath>
+#include <type_traits>
 
 #include "ppf_device.cuh"
 #include "ppf_internal.h"
@@ -43,7 +44,11 @@ __device__ __forceinline__ float to_f32<__nv_bfloat16>(__nv_bfloat16 v) { return
 template <>
 __device__ __forceinline__ float to_f32<__half>(__half v) { return __half2float(v); }
 
-template <typename T>
+// I: the pair index, uint32_t unless a frame has more than LAST_32 pairs (the
+// loop steps past the last pair before it ends)
+constexpr int64_t LAST_32 = 0xFFFFFFFFll - 4096 * 256;
+
+template <typename T, typename I>
 __global__ void prepare_frame_kernel(const T *__restrict__ Z, float *__restrict__ Zp, int W, int H, int Wp,
                                      int Hp, int pad, float bg, DevSummary *sum, int force,
                                      uint32_t *__restrict__ bin_tot, int nbins)
@@ -60,13 +65,13 @@ __global__ void prepare_frame_kernel(const T *__restrict__ Z, float *__restrict_
             bin_tot[t] = 0u;
     // pixel pairs: element (row, col) = (Zb(row, col), Zb(row, col + 1)) with
     // Zb = Z - bg inside the image and 0 in the border of `pad` (pitch Wp)
-    const int n = Wp * Hp;
+    const I n = (I)Wp * (I)Hp, wp = (I)Wp;
     auto px_at = [&](int py, int px) -> float {
         return (px >= 0 && px < W && py >= 0 && py < H) ? to_f32<T>(Z[(int64_t)py * W + px]) - bg : 0.0f;
     };
     float2 *__restrict__ out = reinterpret_cast<float2 *>(Zp);
-    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += gridDim.x * blockDim.x) {
-        const int py = idx / Wp - pad, px = idx % Wp - pad;
+    for (I idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += gridDim.x * blockDim.x) {
+        const int py = (int)(idx / wp) - pad, px = (int)(idx % wp) - pad;
         out[idx] = make_float2(px_at(py, px), px_at(py, px + 1));
     }
 }
@@ -422,9 +427,10 @@ __global__ void cell_map_kernel(PatchGeom geom, KcArr kc, float2 *__restrict__ l
     pdl_trigger();
     constexpr int P = 2 * R + 1;
     geom.Kc = kc.v;
-    const int lw = geom.W + 2 * R, lh = geom.H + 2 * R;
-    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < lw * lh; idx += gridDim.x * blockDim.x) {
-        const int cx = idx % lw - R, cy = idx / lw - R;
+    // (at most 2^31 cells, so the last step stays in 32 unsigned bits)
+    const uint32_t lw = geom.W + 2 * R, lh = geom.H + 2 * R;
+    for (uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x; idx < lw * lh; idx += gridDim.x * blockDim.x) {
+        const int cx = (int)(idx % lw) - R, cy = (int)(idx / lw) - R;
         int ax, ay;
         float gx[P], gy[P], C, l;
         const bool inside = patch_setup<R>(geom, (float)cx, (float)cy, 1.0f, ax, ay, gx, gy, C, &l);
@@ -433,9 +439,9 @@ __global__ void cell_map_kernel(PatchGeom geom, KcArr kc, float2 *__restrict__ l
 }
 
 template <int R>
-static void launch_cell_map_r(const PatchGeom &g, const KcArr &kc, float2 *lmap, int n, cudaStream_t s)
+static void launch_cell_map_r(const PatchGeom &g, const KcArr &kc, float2 *lmap, int64_t n, cudaStream_t s)
 {
-    const int grid = (n + 255) / 256 < 2048 ? (n + 255) / 256 : 2048;
+    const int grid = (n + 255) / 256 < 2048 ? (int)((n + 255) / 256) : 2048;
     launch_pdl(cell_map_kernel<R>, grid, 256, 0, s, g, kc, lmap);
 }
 
@@ -448,7 +454,7 @@ cudaError_t launch_cell_map(ppf_ctx *c)
     KcArr kc;
     for (int k = 0; k < MAX_RADIUS; ++k)
         kc.v[k] = (float)exp(-(2.0 * k + 1.0) * (double)g.inv2s2);
-    const int n = (c->m.width + 2 * R) * (c->m.height + 2 * R);
+    const int64_t n = (int64_t)(c->m.width + 2 * R) * (c->m.height + 2 * R);
     switch (R) {
     case 0: launch_cell_map_r<0>(g, kc, c->lmap, n, c->stream); break;
     case 1: launch_cell_map_r<1>(g, kc, c->lmap, n, c->stream); break;
@@ -486,10 +492,17 @@ cudaError_t launch_prepare_frame(ppf_ctx *c, const void *frame)
         launch_pdl(kernel, grid, 256, 0, c->stream, z, c->Zp, c->m.width, c->m.height, c->Wp, c->Hp, c->pad, bg, c->sum,
                    force, c->bin_tot, c->bin_nbins);
     };
+    auto of = [&](auto *z) {
+        using T = std::remove_cv_t<std::remove_pointer_t<decltype(z)>>;
+        if (n <= LAST_32)
+            go(prepare_frame_kernel<T, uint32_t>, z);
+        else
+            go(prepare_frame_kernel<T, uint64_t>, z);
+    };
     switch (c->m.frame_dtype) {
-    case PPF_BF16: go(prepare_frame_kernel<__nv_bfloat16>, (const __nv_bfloat16 *)frame); break;
-    case PPF_F16: go(prepare_frame_kernel<__half>, (const __half *)frame); break;
-    default: go(prepare_frame_kernel<float>, (const float *)frame);
+    case PPF_BF16: of((const __nv_bfloat16 *)frame); break;
+    case PPF_F16: of((const __half *)frame); break;
+    default: of((const float *)frame);
     }
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && c->lmap)
