@@ -204,8 +204,9 @@ ppf_status ppf_estimate_async(ppf_ctx *ctx, ppf_estimate_t *out_host);
  * Enqueued on the context's stream. */
 ppf_status ppf_get_particles(ppf_ctx *ctx, float *state_dev, int32_t *anc_dev, float *lw_prev_dev);
 
-/* Replaces the current particles (test and restart hook), enqueued on the
- * context's stream; the buffers are copied:
+/* Replaces the current particles (test and restart hook) on the context's
+ * stream; the buffers are copied and the call waits for that, so they may be
+ * reused on return:
  *   state_dev   6 x N float32 SoA, required,
  *   anc_dev     ancestors for the next step, NULL = identity,
  *   lw_prev_dev N float32 starting log-weights for the next step; NULL means

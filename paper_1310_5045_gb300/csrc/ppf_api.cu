@@ -502,8 +502,7 @@ ppf_status ppf_set_particles(ppf_ctx *c, const float *state_dev, const int32_t *
     }
     // particles of unknown spread: the next step bins them (and measures)
     CK(ppf::launch_restart(c, !anc_dev));
-    if (c->bin_key)  // callers may reuse their buffers on return
-        CK(cudaStreamSynchronize(c->stream));
+    CK(cudaStreamSynchronize(c->stream));  // callers may reuse their buffers on return
     c->weighted = false;
     return PPF_OK;
 }
