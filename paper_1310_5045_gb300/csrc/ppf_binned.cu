@@ -440,6 +440,7 @@ __global__ void __launch_bounds__(BinShape<WIDE>::THREADS, BinShape<WIDE>::BLOCK
                 an[e] = ok ? u | (atomicAdd(&hist[u], 1u) << 16) : 0xFFFFFFFFu;
             }
             __syncthreads();
+            int sorted = cntj;
             // exclusive prefix of the T x T counts
             {
                 const int na = a.T * a.T, per = (na + blockDim.x - 1) / blockDim.x, u0 = threadIdx.x * per;
@@ -448,6 +449,9 @@ __global__ void __launch_bounds__(BinShape<WIDE>::THREADS, BinShape<WIDE>::BLOCK
                     sm += hist[u];
                 uint64_t tot;
                 uint64_t run = block_excl_scan_u64(sm, red, &tot);
+                // (the debug build: without the records its anchor check left out)
+                if (!PPF_DCHECK(tot == (uint64_t)cntj, &sum->flags, FLAG_INTERNAL))
+                    sorted = (int)tot;
                 for (int u = u0; u < u0 + per && u < na; ++u) {
                     const uint32_t c = hist[u];
                     hist[u] = (uint32_t)run;
@@ -460,7 +464,7 @@ __global__ void __launch_bounds__(BinShape<WIDE>::THREADS, BinShape<WIDE>::BLOCK
                 if (an[e] != 0xFFFFFFFFu)
                     srt[hist[an[e] & 0xFFFFu] + (an[e] >> 16)] = (uint16_t)(threadIdx.x + e * blockDim.x);
             __syncthreads();
-            for (int j = threadIdx.x; j < cntj; j += blockDim.x) {
+            for (int j = threadIdx.x; j < sorted; j += blockDim.x) {
                 const uint32_t r = srt[j];
                 const float4 v = rb[r];
                 int cx, cy;
