@@ -170,18 +170,19 @@ __host__ __device__ inline int scale_bits(int64_t n)
 // 2^f for f in [0, 1): Taylor polynomial of e^(f ln 2) to degree 9, the
 // coefficients (ln 2)^n / n! rounded to float32, evaluated by Horner's rule
 // with fused multiply-adds.
-__device__ __forceinline__ float exp2_frac(float f)
+__device__ __forceinline__ float2 exp2_frac2(float2 f)
 {
-    float p = 0x1.b5253ep-24f;
-    p = __fmaf_rn(p, f, 0x1.62c022p-20f);
-    p = __fmaf_rn(p, f, 0x1.ffcbfcp-17f);
-    p = __fmaf_rn(p, f, 0x1.430912p-13f);
-    p = __fmaf_rn(p, f, 0x1.5d87fep-10f);
-    p = __fmaf_rn(p, f, 0x1.3b2ab6p-7f);
-    p = __fmaf_rn(p, f, 0x1.c6b08ep-5f);
-    p = __fmaf_rn(p, f, 0x1.ebfbep-3f);
-    p = __fmaf_rn(p, f, 0x1.62e43p-1f);
-    p = __fmaf_rn(p, f, 1.0f);
+    auto c = [](float v) { return make_float2(v, v); };
+    float2 p = c(0x1.b5253ep-24f);
+    p = __ffma2_rn(p, f, c(0x1.62c022p-20f));
+    p = __ffma2_rn(p, f, c(0x1.ffcbfcp-17f));
+    p = __ffma2_rn(p, f, c(0x1.430912p-13f));
+    p = __ffma2_rn(p, f, c(0x1.5d87fep-10f));
+    p = __ffma2_rn(p, f, c(0x1.3b2ab6p-7f));
+    p = __ffma2_rn(p, f, c(0x1.c6b08ep-5f));
+    p = __ffma2_rn(p, f, c(0x1.ebfbep-3f));
+    p = __ffma2_rn(p, f, c(0x1.62e43p-1f));
+    p = __ffma2_rn(p, f, c(1.0f));
     return p;
 }
 
@@ -214,36 +215,9 @@ __device__ __forceinline__ uint64_t quantise_tail(uint32_t rb, float p, int s)
     return shr_u64(X, n);
 }
 
-__device__ __forceinline__ uint64_t quantise(float lw, float M, int s)
-{
-    const float d = __fsub_rn(lw, M);
-    const float t = fmaxf(__fmul_rn(d, 0x1.715476p+0f), -64.0f);
-    const float r = __fadd_rd(t, FLOOR_MAGIC);
-    const float f = __fsub_rn(t, __fsub_rn(r, FLOOR_MAGIC));
-    return quantise_tail(__float_as_uint(r), exp2_frac(f), s);
-}
-
-// exp2_frac of two values at once: the same Horner steps as packed two-lane
-// FMAs, each lane rounding as the scalar form.
-__device__ __forceinline__ float2 exp2_frac2(float2 f)
-{
-    auto c = [](float v) { return make_float2(v, v); };
-    float2 p = c(0x1.b5253ep-24f);
-    p = __ffma2_rn(p, f, c(0x1.62c022p-20f));
-    p = __ffma2_rn(p, f, c(0x1.ffcbfcp-17f));
-    p = __ffma2_rn(p, f, c(0x1.430912p-13f));
-    p = __ffma2_rn(p, f, c(0x1.5d87fep-10f));
-    p = __ffma2_rn(p, f, c(0x1.3b2ab6p-7f));
-    p = __ffma2_rn(p, f, c(0x1.c6b08ep-5f));
-    p = __ffma2_rn(p, f, c(0x1.ebfbep-3f));
-    p = __ffma2_rn(p, f, c(0x1.62e43p-1f));
-    p = __ffma2_rn(p, f, c(1.0f));
-    return p;
-}
-
-// quantise of two weights: the float32 steps as packed two-lane operations
-// (a - M as a + (-M), exact in IEEE arithmetic), so both results equal the
-// scalar quantise bit for bit.
+// The fixed-point weights of two log-weights: every float32 step as one packed
+// two-lane operation, each lane rounding as the scalar step does (lw - M as
+// lw + (-M), the same in IEEE arithmetic).
 __device__ __forceinline__ void quantise2(float a, float b, float M, int s, uint64_t &qa, uint64_t &qb)
 {
     const float2 magic = make_float2(FLOOR_MAGIC, FLOOR_MAGIC);
@@ -352,14 +326,6 @@ __device__ __forceinline__ float warp_max(float v)
 }
 
 __device__ __forceinline__ float warp_sum(float v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-__device__ __forceinline__ double warp_sum_d(double v)
 {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)

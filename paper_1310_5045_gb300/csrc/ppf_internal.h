@@ -136,10 +136,9 @@ struct Scratch {
     GroupGrid *ggrid;  // [G]  two-stage RPA: every group's draw
     int32_t *split;    // [4 (T + G + 2 N / ITEM_TICKETS + 2)] two-stage RPA: extra work items (tile or -1, group, run, 0)
     // scheduler (RPA)
-    uint64_t *skey;    // [2G] sort / merge buffers
-    int64_t *sval;     // [5G]
-    int32_t *seg_src;  // segments: ticket start, slot start, length, chunk prefix
-    int64_t *seg_tick;
+    uint64_t *skey;    // [2G] the schedule's sort keys
+    int64_t *sval;     // [2G] LGS: sent and received per group
+    int64_t *seg_tick;  // [2G+1] segments: ticket start, slot start, length, chunk prefix
     int64_t *seg_dst;
     int64_t *seg_len;
     int32_t *seg_chunk; // [2G+1]

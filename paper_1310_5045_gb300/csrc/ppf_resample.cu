@@ -629,11 +629,10 @@ struct SchedArgs {
     int64_t *goff_new;
     const int64_t *Tg;
     uint64_t *key;      // [2 * G]  (sender keys, receiver keys)
-    int64_t *val;       // [5 * G]  (PS, PR, sent, recv, merge buffer)
+    int64_t *val;       // [2 * G]  (sent, received; LGS)
     int32_t *seg_chunk; // [2G + 2]
     int64_t *seg_tick, *seg_dst, *seg_len;  // [2G + 1]
     DevSummary *sum;
-    int links_only;  // the fill wrote the kept segments already: copy work items for the links only
     Balanced bl;     // the balanced targets n_g
 };
 
@@ -747,8 +746,6 @@ __device__ void schedule_small(const SchedArgs &A, unsigned char *mem)
                     }
                 }
                 if (j >= 64 || (j == 1 && k >= 64))
-                    __syncthreads();
-                else if (j > 32)
                     __syncthreads();
                 else
                     __syncwarp();
@@ -1329,33 +1326,6 @@ __device__ void block_sort_u64(uint64_t *g, int n, uint64_t *sm, int cap)
     __syncthreads();
 }
 
-// first index in sorted a[0..n) with a[i] > v
-__device__ __forceinline__ int upper_bound_i64(const int64_t *a, int n, int64_t v)
-{
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (a[mid] > v)
-            hi = mid;
-        else
-            lo = mid + 1;
-    }
-    return lo;
-}
-
-__device__ __forceinline__ int lower_bound_i64(const int64_t *a, int n, int64_t v)
-{
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (a[mid] < v)
-            lo = mid + 1;
-        else
-            hi = mid;
-    }
-    return lo;
-}
-
 __device__ __forceinline__ int lower_bound_i32(const int32_t *a, int n, int32_t v)
 {
     int lo = 0, hi = n;
@@ -1503,9 +1473,9 @@ __device__ void schedule_links_balanced(const SchedArgs &A, int nS, int nR, bool
 
 __global__ void __launch_bounds__(1024) schedule_kernel(SchedArgs A)
 {
-    extern __shared__ uint64_t sm[];   // sort_smem_bytes(G) (GS: G words)
+    extern __shared__ uint64_t sm[];   // sched_smem_bytes(G)
     __shared__ uint64_t red[33];
-    __shared__ int nS_s, nR_s, L_s;
+    __shared__ int nS_s, nR_s;
     const int32_t G = A.G;
     DevSummary *sum = A.sum;
     if (sum->degenerate) {
@@ -1519,7 +1489,6 @@ __global__ void __launch_bounds__(1024) schedule_kernel(SchedArgs A)
         return;
     }
     uint64_t *Skey = A.key, *Rkey = A.key + G;
-    int64_t *PS = A.val, *PR = A.val + G;
     // 1. senders / receivers, compacted in group order.  key = amount << 24 | g
     //    (amount <= N < 2^31 fits 40 bits; g < 2^24).  For sorting by amount
     //    descending then g ascending we sort ((2^40-1-amount) << 24 | g).
@@ -1571,35 +1540,25 @@ __global__ void __launch_bounds__(1024) schedule_kernel(SchedArgs A)
         block_sort_u64(Skey, nS, sm, G);
         block_sort_u64(Rkey, nR, sm, G);
     }
-    if (A.links_only) {
+    if (A.scheme != PPF_RPA_LGS) {  // the fill wrote the kept tickets already
         schedule_links_balanced(A, nS, nR, sorted, sm, red);
         return;
     }
-    auto amount = [&](uint64_t k) -> int64_t {
-        return sorted ? (int64_t)(0xFFFFFFFFFFull - (k >> 24)) : (int64_t)(k >> 24);
-    };
+    auto amount = [&](uint64_t k) -> int64_t { return (int64_t)(0xFFFFFFFFFFull - (k >> 24)); };
     auto group = [&](uint64_t k) -> int32_t { return (int32_t)(k & 0xFFFFFFull); };
     // per-group sent / received totals
-    int64_t *sent = A.val + 2 * G, *recv = A.val + 3 * G;
+    int64_t *sent = A.val, *recv = A.val + G;
     for (int g = threadIdx.x; g < G; g += blockDim.x) {
         sent[g] = 0;
         recv[g] = 0;
     }
     __syncthreads();
-    int L = 0;
-    if (A.scheme == PPF_RPA_LGS) {
-        L = nS < nR ? nS : nR;
-        for (int i = threadIdx.x; i < L; i += blockDim.x) {
-            const int64_t a = amount(Skey[i]), b = amount(Rkey[i]);
-            const int64_t c = a < b ? a : b;
-            sent[group(Skey[i])] = c;
-            recv[group(Rkey[i])] = c;
-        }
-    } else {
-        for (int i = threadIdx.x; i < nS; i += blockDim.x)
-            sent[group(Skey[i])] = amount(Skey[i]);
-        for (int i = threadIdx.x; i < nR; i += blockDim.x)
-            recv[group(Rkey[i])] = amount(Rkey[i]);
+    const int L = nS < nR ? nS : nR;
+    for (int i = threadIdx.x; i < L; i += blockDim.x) {
+        const int64_t a = amount(Skey[i]), b = amount(Rkey[i]);
+        const int64_t c = a < b ? a : b;
+        sent[group(Skey[i])] = c;
+        recv[group(Rkey[i])] = c;
     }
     __syncthreads();
     // 2. new sizes and offsets: m'_g = o_g - sent_g + recv_g
@@ -1649,83 +1608,16 @@ __global__ void __launch_bounds__(1024) schedule_kernel(SchedArgs A)
         seg_len[g] = (A.Tg[g + 1] - A.Tg[g]) - sent[g];
     }
     // 4. links
-    if (A.scheme == PPF_RPA_LGS) {
-        for (int i = threadIdx.x; i < L; i += blockDim.x) {
-            const int32_t s = group(Skey[i]), r = group(Rkey[i]);
-            const int64_t c = sent[s];
-            const int64_t keep_s = (A.Tg[s + 1] - A.Tg[s]) - c;
-            const int64_t keep_r = A.Tg[r + 1] - A.Tg[r];
-            seg_tick[G + i] = A.Tg[s] + keep_s;
-            seg_dst[G + i] = off[r] + keep_r;
-            seg_len[G + i] = c;
-        }
-        if (threadIdx.x == 0)
-            L_s = L;
-        __syncthreads();
-    } else {
-        // prefix sums of the amounts in list order (inclusive)
-        for (int i = threadIdx.x; i < nS; i += blockDim.x)
-            PS[i] = amount(Skey[i]);
-        for (int i = threadIdx.x; i < nR; i += blockDim.x)
-            PR[i] = amount(Rkey[i]);
-        __syncthreads();
-        int64_t d1, d2;
-        block_scan_i64(PS, nS, red, &d1);
-        block_scan_i64(PR, nR, red, &d2);
-        // now PS[i], PR[j] are exclusive starts; piece starts are the union of
-        // both start sets (0 is in both).  Merge them (PS first on ties).
-        int64_t *MG = A.val + 4 * G;  // at most nS + nR <= G entries
-        // the binary searches below run on shared copies of the two prefix
-        // arrays (nS + nR <= G <= MAX_SCHED_GROUPS entries; the sort is done)
-        int64_t *sPS = reinterpret_cast<int64_t *>(sm), *sPR = sPS + nS;
-        __syncthreads();
-        for (int i = threadIdx.x; i < nS; i += blockDim.x)
-            sPS[i] = PS[i];
-        for (int j = threadIdx.x; j < nR; j += blockDim.x)
-            sPR[j] = PR[j];
-        __syncthreads();
-        for (int i = threadIdx.x; i < nS; i += blockDim.x)
-            MG[i + lower_bound_i64(sPR, nR, sPS[i])] = sPS[i];
-        for (int j = threadIdx.x; j < nR; j += blockDim.x)
-            MG[j + upper_bound_i64(sPS, nS, sPR[j])] = sPR[j];
-        __syncthreads();
-        const int nm = nS + nR;
-        // distinct starts -> links; store compacted into seg arrays after G
-        {
-            const int per = (nm + blockDim.x - 1) / blockDim.x;
-            const int i0 = threadIdx.x * per;
-            uint64_t c = 0;
-            for (int k = 0; k < per; ++k) {
-                const int i = i0 + k;
-                if (i < nm && (i == 0 || MG[i] != MG[i - 1]))
-                    ++c;
-            }
-            uint64_t tl;
-            uint64_t pos = block_excl_scan_u64(c, red, &tl);
-            for (int k = 0; k < per; ++k) {
-                const int i = i0 + k;
-                if (i < nm && (i == 0 || MG[i] != MG[i - 1])) {
-                    const int64_t a = MG[i];
-                    const int si = upper_bound_i64(sPS, nS, a) - 1;  // sender piece contains a
-                    const int rj = upper_bound_i64(sPR, nR, a) - 1;
-                    const int64_t se = sPS[si] + amount(Skey[si]);
-                    const int64_t re = sPR[rj] + amount(Rkey[rj]);
-                    const int64_t e = se < re ? se : re;
-                    const int32_t s = group(Skey[si]), r = group(Rkey[rj]);
-                    const int64_t keep_s = (A.Tg[s + 1] - A.Tg[s]) - sent[s];
-                    const int64_t keep_r = A.Tg[r + 1] - A.Tg[r];
-                    seg_tick[G + pos] = A.Tg[s] + keep_s + (a - sPS[si]);
-                    seg_dst[G + pos] = off[r] + keep_r + (a - sPR[rj]);
-                    seg_len[G + pos] = e - a;
-                    ++pos;
-                }
-            }
-            if (threadIdx.x == 0)
-                L_s = (nm > 0) ? (int)tl : 0;
-        }
-        __syncthreads();
+    for (int i = threadIdx.x; i < L; i += blockDim.x) {
+        const int32_t s = group(Skey[i]), r = group(Rkey[i]);
+        const int64_t c = sent[s];
+        const int64_t keep_s = (A.Tg[s + 1] - A.Tg[s]) - c;
+        const int64_t keep_r = A.Tg[r + 1] - A.Tg[r];
+        seg_tick[G + i] = A.Tg[s] + keep_s;
+        seg_dst[G + i] = off[r] + keep_r;
+        seg_len[G + i] = c;
     }
-    L = L_s;
+    __syncthreads();
     const int nseg = G + L;
     // 5. copy work items per segment
     {
@@ -1735,8 +1627,7 @@ __global__ void __launch_bounds__(1024) schedule_kernel(SchedArgs A)
         for (int k = 0; k < per; ++k) {
             const int i = i0 + k;
             if (i < nseg) {
-                if (i >= G || !A.links_only)
-                    c += (uint64_t)((seg_len[i] + COPY_CHUNK - 1) / COPY_CHUNK);
+                c += (uint64_t)((seg_len[i] + COPY_CHUNK - 1) / COPY_CHUNK);
                 if (i >= G)
                     mv += (uint64_t)seg_len[i];
             }
@@ -1748,8 +1639,7 @@ __global__ void __launch_bounds__(1024) schedule_kernel(SchedArgs A)
             const int i = i0 + k;
             if (i < nseg) {
                 A.seg_chunk[i] = (int32_t)run;
-                if (i >= G || !A.links_only)
-                    run += (uint64_t)((seg_len[i] + COPY_CHUNK - 1) / COPY_CHUNK);
+                run += (uint64_t)((seg_len[i] + COPY_CHUNK - 1) / COPY_CHUNK);
             }
         }
         if (threadIdx.x == 0) {
@@ -2288,7 +2178,6 @@ static SchedArgs sched_args(ppf_ctx *c, int scheme, bool two_stage)
     A.seg_dst = c->sc.seg_dst;
     A.seg_len = c->sc.seg_len;
     A.sum = c->sum;
-    A.links_only = A.scheme != PPF_RPA_LGS;
     A.bl = balanced_layout(c->N, c->G);
     return A;
 }
