@@ -266,9 +266,14 @@ __device__ void grad_finalize(const GradPartial *part, int n, DevSummary *sum, i
     }
 }
 
-// (up to R = 5 the kernel fits 128 registers: two blocks per SM)
+// Two blocks per SM (128 registers) up to R = 6, one (254) above, where the
+// second block's 12 to 48 bytes of spills cost more than it hides.  A frame of
+// the gradient with two blocks and with one: R = 6 104.4 and 105.3 us at 2^20
+// particles, 43.1 and 45.7 at 200,000, 30.5 and 31.8 at 50,001; R = 7 122.6 and
+// 120.9, 50.7 and 49.3, 32.6 and 32.9; R = 8 144.3 and 136.8, 56.5 and 53.4,
+// 34.4 and 35.4.
 template <int R>
-__global__ void __launch_bounds__(256, R <= 5 ? 2 : 1) grad_step_kernel(GradArgs a)
+__global__ void __launch_bounds__(256, R <= 6 ? 2 : 1) grad_step_kernel(GradArgs a)
 {
     if (!pdl_wait())
         return;
