@@ -324,7 +324,7 @@ class ParticleFilter:
         size = C.sizeof(_Estimate)
         if out is None:
             out = torch.empty(size, dtype=torch.uint8, pin_memory=True)
-        elif not out.is_contiguous() or out.numel() * out.element_size() < size:
+        elif out.nbytes < size or not out.is_contiguous():
             raise ValueError(f"out must be a contiguous tensor of at least {size} bytes")
         self._check(self.L.ppf_estimate_async(self._ctx, C.c_void_p(out.data_ptr())), "ppf_estimate_async")
         return out

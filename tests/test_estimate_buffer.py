@@ -14,24 +14,27 @@ RULE = r"""
 #include "ppf_mapped.h"
 #include <cstdio>
 #include <initializer_list>
-// host bytes [64, 64 + mapped) of an imaginary address space are mapped `shift` bytes on
+// host bytes [64, end) of an imaginary address space are mapped `shift` bytes on; the pages that hold them are accessible
 int main()
 {
-    for (uintptr_t shift : {uintptr_t(0x1000), uintptr_t(0x1004)})
-        for (uintptr_t p = 56; p < 90; ++p)
-            for (size_t mapped : {size_t(0), size_t(103), size_t(104), size_t(111), size_t(112), size_t(200)}) {
+    const uintptr_t page = 4096;
+    for (uintptr_t shift : {uintptr_t(0x10000), uintptr_t(0x10004)})
+        for (uintptr_t end : {page - 200, page - 8, page, page + 1, page + 96, 2 * page})
+            for (uintptr_t p = page - 240; p < page + 16; ++p) {
                 auto map = [&](void *q) -> void * {
                     const uintptr_t a = (uintptr_t)q;
-                    return a >= 64 && a < 64 + mapped ? (void *)(a + shift) : nullptr;
+                    return a >= 64 && a < end ? (void *)(a + shift) : nullptr;
                 };
-                const bool ok = p % 8 == 0 && shift % 8 == 0 && p >= 64 && p + 104 <= 64 + mapped;
-                void *want = ok ? (void *)(p + shift) : nullptr;
-                if (ppf::mapped_words((void *)p, 104, map) != want)
-                    return std::printf("shift %zx p %zu mapped %zu\n", (size_t)shift, (size_t)p, mapped), 1;
+                void *got = ppf::mapped_words((void *)p, 104, map);
+                const bool aligned = p % 8 == 0 && shift % 8 == 0, reachable = p + 104 <= (end + page - 1) / page * page;
+                if (got && (got != (void *)(p + shift) || !aligned || !reachable))
+                    return std::printf("handed out: shift %zx p %zu end %zu\n", (size_t)shift, (size_t)p, (size_t)end), 1;
+                if (!got && aligned && p + 104 <= end)
+                    return std::printf("kept back: shift %zx p %zu end %zu\n", (size_t)shift, (size_t)p, (size_t)end), 1;
             }
-    // the last byte in another mapping than the first
-    auto split = [](void *q) -> void * { return (void *)((uintptr_t)q + ((uintptr_t)q < 128 ? 0x1000 : 0x2000)); };
-    return ppf::mapped_words((void *)64, 104, split) != nullptr;
+    // the last byte on another page and in another mapping than the first
+    auto split = [=](void *q) -> void * { return (void *)((uintptr_t)q + ((uintptr_t)q < page ? 0x10000 : 0x20000)); };
+    return ppf::mapped_words((void *)(page - 48), 104, split) != nullptr;
 }
 """
 
