@@ -413,7 +413,7 @@ ppf_status ppf_fp32_peak(int32_t packed, int32_t repeats, double *tflops_out, do
  *   anc_dev    n int32 (device, caller-owned): ancestor of every slot; the
  *              identity when every weight is zero or NaN.
  *   cuda_stream stream to enqueue on (NULL = legacy default stream).
- * The scratch array (about 391 KB) lives on every device that loads the
+ * The scratch array (about 395 KB) lives on every device that loads the
  * library until the process exits.  The first call on a device looks up its
  * address (with that device current), and so does the first call after the
  * device's context changed (a cudaDeviceReset); make those calls before any

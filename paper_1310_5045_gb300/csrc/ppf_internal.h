@@ -210,10 +210,14 @@ enum Phase { PH_PREPARE = 0, PH_STEP = 1, PH_FINALIZE = 2, PH_RESAMPLE = 3 };
 // is still running (programmatic dependent launch).  The kernel begins with
 // pdl_wait(), then pdl_trigger(): it reads nothing the previous kernel writes
 // before that kernel is complete, and every kernel of a chain has seen the one
-// before complete, so a kernel after it sees them all.  All kernels of a step
-// and a resampling are launched this way: what is hidden is the launch, 2 to 3
-// us of a frame's 7 to 10 kernels each (a frame of 1,000,003 particles: 102 us
-// with plain launches, 81 with these; 2^20 particles of the gradient: 74 and 64).
+// before complete, so a kernel after it sees them all.  What is hidden is the
+// launch, 2 to 3 us of a frame's 7 to 10 kernels each (a frame of 1,000,003
+// particles: 102 us with plain launches, 81 with these; 2^20 particles of the
+// gradient: 74 and 64).  The kernels of a step, a resampling, the gradient and
+// a batched frame are launched this way, except group_grid_kernel, and the
+// schedule on the side stream and the routing copy that joins it (both behind
+// an event).  The initial draw, the read-out and the allocation-free draw's
+// clear, maximum and identity are plain launches too.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s, Args &&...args)
 {

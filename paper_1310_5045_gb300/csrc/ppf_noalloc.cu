@@ -41,7 +41,8 @@ constexpr size_t OFF_TT = align256(OFF_CT + sizeof(uint64_t) * (NOALLOC_MAX_T + 
 constexpr size_t OFF_EX = align256(OFF_TT + sizeof(int64_t) * (NOALLOC_MAX_T + 1));  // further runs (int2)
 constexpr size_t OFF_TO = align256(OFF_EX + sizeof(int2) * (NOALLOC_MAX_N / ITEM_TICKETS + 1));
 constexpr size_t OFF_ST = align256(OFF_TO + sizeof(int32_t) * NOALLOC_MAX_T);
-constexpr size_t SCRATCH_BYTES = align256(OFF_ST + sizeof(uint64_t) * STRIPS * NOALLOC_MAX_T);  // ~391 KB
+constexpr size_t SCRATCH_BYTES = align256(OFF_ST + sizeof(uint64_t) * STRIPS * NOALLOC_MAX_T);
+static_assert(SCRATCH_BYTES <= 395000, "the header states about 395 KB");
 
 static __device__ __align__(256) unsigned char g_scratch[SCRATCH_BYTES];
 

@@ -1762,7 +1762,9 @@ struct EmitRing {
 // The draw of a group larger than the block's 16 NT particles, in chunks of
 // them; the tickets of a chunk are [T(carry), T(carry + total)), T the count
 // below of the group's sz tickets.  (A call: its registers stay out of the
-// kernel's common path.)
+// kernel's common path.)  The weights are read three times, and 284 to 448 bytes
+// a thread spill: a frame of RNA at 2,000,000 particles takes 72.7 us in groups
+// of 4096, 87.5 in groups of 5000 and 98.4 in groups of 16384.
 template <int NT>
 static __device__ __noinline__ void rna_chunks(const float *__restrict__ lw, int64_t N, int64_t lo, int64_t sz, float Mg,
                                                int s, TicketGrid tg, TicketScale sc, ParentSmemT<NT> *sm, EmitRing em)
